@@ -63,8 +63,8 @@ struct FitArgs {
   const int *win_off;      // [n_win] slot offset within a series
   const int *n_valid;      // [n_dm][n_win]
   int S_tot;
-  int tile;                // list mode: rows per CTA
-  int TT;                  // implicit layout: APs per time tile (one CTA per DM, tile, baseline)
+  int tile;                // list mode: rows per CTA (plain launches: at most)
+  int TT;                  // implicit layout: APs per time tile (one CTA per DM, tile, baseline; plain launches: at most)
   // explicit list
   const int *seg;          // [n_seg][4]
   long long n_seg;
@@ -143,6 +143,7 @@ cudaError_t launch_fit_fft(const FitArgs &a, int n_bl, bool list_mode, cudaStrea
 cudaError_t launch_fit_fft_batch(const FitArgs &a, const BatchScan *scans_dev, int n_scans, long long total_items,
                                  unsigned int *counter, int ctas_per_sm, cudaStream_t st, int64_t *launches);
 size_t max_smem_optin();
+int sm_count();
 bool fit_grid(const FitArgs &a, int n_bl, bool list_mode, dim3 *grid);
 
 // kernels_tree.cu: multi-window fit through the additivity of the delay-resolution matrix

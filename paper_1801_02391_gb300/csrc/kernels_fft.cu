@@ -5,9 +5,13 @@
 //  MBD: with g = 32 g1 + g2 and q = q1 + (Lm/32) q2,
 //       G(m, q) = sum_g2 w32^(g2 q2) [ sum_{n: g_n = g2 mod 32} Y(n, m) wLm^(g_n q1) ]
 //
-// One CTA of 128 threads fits a tile of segments one after the other: gather into shared
+// One CTA fits a tile of segments one after the other: gather into shared
 // memory, one SBD task (n, m1) per thread, then Ls * Lm / 32 MBD tasks (m, q1) that each end
-// in a 32-point register FFT and the maximum of its 32 cells.  The channel of each residue
+// in a 32-point register FFT and the maximum of its 32 cells.  CTAs have 128 threads, four on an
+// SM, so one's gather runs beside another's transforms; a list too short to give every SM its
+// four CTAs runs one 512-thread CTA per segment instead (the MBD tasks of a segment, 2048 on the
+// four-band grid, are most of its latency): a call with 40 segments 846 -> 92 us, against 16 of them
+// one after the other in a 128-thread CTA.  The channel of each residue
 // class g2 comes from the kernel parameters (uniform across the CTA), so the MBD inner sum is
 // unrolled over the occupied channels only.  The per-task maximum packs the cell's q2 into the
 // 6 low mantissa bits of |G|^2 (a 2^-17 relative truncation) and takes an integer max.
@@ -16,7 +20,10 @@
 
 namespace frbx {
 
-constexpr int kFftThreads = 128;
+constexpr int kFftThreads = 128;      // four CTAs per SM
+constexpr int kFftWideThreads = 512;  // one CTA per SM: a list shorter than the GPU
+constexpr int kFftWarps = kFftWideThreads / 32;
+constexpr int kFftWideRows = 2;       // longest list of the wide form, in segments per SM
 
 struct FftSmem {
   int xs, ys, ts;
@@ -31,12 +38,12 @@ __host__ __device__ inline FftSmem fft_smem_layout(int N, int Ls, int Lm, int J1
   l.ts = JP + 1;
   l.bytes = sizeof(float2) * ((size_t)N * l.xs + (size_t)N * l.ys + (size_t)(Ls / 32) * l.ts +
                               (size_t)N * (Lm / 32)) +
-            16 * sizeof(int);  // block reduction (4 warps)
+            2 * kFftWarps * sizeof(int);  // block reduction
   return l;
 }
 
-template <int OCC, bool kFull, bool kBatch>
-__global__ void __launch_bounds__(kFftThreads, 4)
+template <int OCC, bool kFull, bool kBatch, int kThreads = kFftThreads>
+__global__ void __launch_bounds__(kThreads, 512 / kThreads)
     k_fit_fft(const __grid_constant__ FitArgs a, int list, const BatchScan *scans, int n_scans, long long total,
               unsigned int *counter) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -50,7 +57,7 @@ __global__ void __launch_bounds__(kFftThreads, 4)
   float2 *stw = Y + N * L.ys;                    // [PS][ts]
   float2 *mtw = stw + PS * L.ts;                 // [N][PM]
   float *rp = reinterpret_cast<float *>(mtw + N * PM);
-  int *ri = reinterpret_cast<int *>(rp + 8);
+  int *ri = reinterpret_cast<int *>(rp + kFftWarps);
 
   for (int i = threadIdx.x; i < N * L.xs; i += blockDim.x) X[i] = make_float2(0.f, 0.f);
   for (int i = threadIdx.x; i < PS * JP; i += blockDim.x) {
@@ -149,14 +156,14 @@ void set_fft_constants() {
 
 bool fft_supported(int Ls, int Lm, int J) { return Ls % 32 == 0 && Lm % 32 == 0 && J <= Ls; }
 
-template <int OCC, bool kFull, bool kBatch>
+template <int OCC, bool kFull, bool kBatch, int kThreads = kFftThreads>
 static cudaError_t launch_one(const FitArgs &a, dim3 grid, size_t smem, int list, cudaStream_t st,
                               const BatchScan *scans = nullptr, int n_scans = 0, long long total = 0,
                               unsigned int *counter = nullptr) {
-  cudaError_t e = cudaFuncSetAttribute(k_fit_fft<OCC, kFull, kBatch>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  auto kern = k_fit_fft<OCC, kFull, kBatch, kThreads>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_fit_fft<OCC, kFull, kBatch><<<grid, kFftThreads, smem, st>>>(a, list, scans, n_scans, total, counter);
+  kern<<<grid, kThreads, smem, st>>>(a, list, scans, n_scans, total, counter);
   return cudaGetLastError();
 }
 
@@ -170,7 +177,12 @@ cudaError_t launch_fit_fft(const FitArgs &a, int n_bl, bool list_mode, cudaStrea
   const bool full = a.m_lo == 0 && a.m_len == a.Ls && a.q_lo == 0 && a.q_len == a.Lm;
   const int list = list_mode ? 1 : 0;
   cudaError_t e;
-  if (a.occ == 1) e = full ? launch_one<1, true, false>(a, grid, smem, list, st) : launch_one<1, false, false>(a, grid, smem, list, st);
+  // one segment per CTA and no more than kFftWideRows per SM: the wide form
+  const bool wide = list_mode && a.tile == 1 && a.n_seg <= (long long)kFftWideRows * sm_count();
+  if (wide && a.occ == 1) e = full ? launch_one<1, true, false, kFftWideThreads>(a, grid, smem, list, st) : launch_one<1, false, false, kFftWideThreads>(a, grid, smem, list, st);
+  else if (wide && a.occ == 2) e = full ? launch_one<2, true, false, kFftWideThreads>(a, grid, smem, list, st) : launch_one<2, false, false, kFftWideThreads>(a, grid, smem, list, st);
+  else if (wide) e = full ? launch_one<4, true, false, kFftWideThreads>(a, grid, smem, list, st) : launch_one<4, false, false, kFftWideThreads>(a, grid, smem, list, st);
+  else if (a.occ == 1) e = full ? launch_one<1, true, false>(a, grid, smem, list, st) : launch_one<1, false, false>(a, grid, smem, list, st);
   else if (a.occ == 2) e = full ? launch_one<2, true, false>(a, grid, smem, list, st) : launch_one<2, false, false>(a, grid, smem, list, st);
   else e = full ? launch_one<4, true, false>(a, grid, smem, list, st) : launch_one<4, false, false>(a, grid, smem, list, st);
   ++*launches;
@@ -183,11 +195,8 @@ cudaError_t launch_fit_fft_batch(const FitArgs &a, const BatchScan *scans, int n
   const size_t smem = fft_smem_layout(a.N, a.Ls, a.Lm, a.J1).bytes;
   if (smem > max_smem_optin()) return cudaErrorInvalidConfiguration;
   if (total <= 0) return cudaSuccess;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int per_sm = ctas_per_sm > 0 ? ctas_per_sm : 4;
-  const dim3 grid((unsigned)(sms * per_sm));
+  const dim3 grid((unsigned)(sm_count() * per_sm));
   const bool full = a.m_lo == 0 && a.m_len == a.Ls && a.q_lo == 0 && a.q_len == a.Lm;
   cudaError_t e;
   if (a.occ == 1) e = full ? launch_one<1, true, true>(a, grid, smem, 0, st, scans, n_scans, total, counter) : launch_one<1, false, true>(a, grid, smem, 0, st, scans, n_scans, total, counter);
