@@ -1423,29 +1423,22 @@ extern "C" int frbx_calibrate(frbx_handle *h, const void *vis, int32_t vis_on_de
   int rc = check_vis(h, vis, vis_on_device, n_bl, T, st, &dvis);
   if (rc) return rc;
   const int C = h->C, N = h->N;
-  // scratch: FP64 sums, complex64 copy, unit weights, zero shifts, rows, fits, delays
+  // scratch: FP64 sums, complex64 copy, unit weights, zero shifts, rows, fits, then the outputs in
+  // one stretch (SBD, MBD, delays, phases), copied to the host at once
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t o = off;
     off = (off + bytes + 255) & ~(size_t)255;
     return o;
   };
+  const size_t n_out = (size_t)n_bl * (2 + 2 * N);
   const size_t o_xs = take(16 * (size_t)n_bl * C), o_xc = take(8 * (size_t)n_bl * C), o_w = take(8 * (size_t)C),
                o_dk = take(4 * (size_t)C), o_rows = take(16 * (size_t)n_bl), o_fit = take(8 * (size_t)n_bl),
-               o_sm = take(16 * (size_t)n_bl), o_d = take(8 * (size_t)n_bl * N), o_p = take(8 * (size_t)n_bl * N);
+               o_out = take(8 * n_out);
   FRBX_CK(h, ensure(h, h->calib, off));
   unsigned char *b = (unsigned char *)h->calib.p;
   FRBX_CK(h, frbx::launch_cal_sum(dvis, T, C, n_bl, k0, l, h->d_wrot, (double2 *)(b + o_xs), (float2 *)(b + o_xc),
-                                  (float2 *)(b + o_w), st, &h->launches));
-  FRBX_CK(h, cudaMemsetAsync(b + o_dk, 0, 4 * (size_t)C, st));
-  std::vector<int32_t> rows((size_t)4 * n_bl);
-  for (int i = 0; i < n_bl; ++i) {
-    rows[4 * i] = i;
-    rows[4 * i + 1] = 0;
-    rows[4 * i + 2] = 1;
-    rows[4 * i + 3] = 0;
-  }
-  FRBX_CK(h, cudaMemcpyAsync(b + o_rows, rows.data(), 16 * (size_t)n_bl, cudaMemcpyHostToDevice, st));
+                                  (float2 *)(b + o_w), (int *)(b + o_dk), (int4 *)(b + o_rows), st, &h->launches));
   // (c) common fringe fit on the grid, no calibration rotation
   FitArgs a{};
   fill_fit_tables(h, &a, (const float2 *)(b + o_xc), 1, 1);
@@ -1462,26 +1455,19 @@ extern "C" int frbx_calibrate(frbx_handle *h, const void *vis, int32_t vis_on_de
   cudaError_t e = frbx::launch_fit(a, n_bl, true, 0, st, &h->launches);
   if (e == cudaErrorInvalidConfiguration) return fail(h, FRBX_EUNSUPPORTED, "fit kernel does not fit this shape");
   FRBX_CK(h, e);
-  std::vector<frbx_seg> fits((size_t)n_bl);
-  FRBX_CK(h, cudaMemcpyAsync(fits.data(), b + o_fit, 8 * (size_t)n_bl, cudaMemcpyDeviceToHost, st));
-  FRBX_CK(h, cudaStreamSynchronize(st));
-  std::vector<double> sm((size_t)2 * n_bl);
-  for (int i = 0; i < n_bl; ++i) {
-    const int m = fits[(size_t)i].sbd_idx, q = fits[(size_t)i].mbd_idx;
-    const int sm_ = m < h->Ls / 2 ? m : m - h->Ls, sq = q < h->Lm / 2 ? q : q - h->Lm;
-    sm[(size_t)2 * i] = (((double)sm_ * h->J) * 1000.0) / ((double)h->Ls * h->f_bw);
-    sm[(size_t)2 * i + 1] = ((double)sq * 1000.0) / ((double)h->Lm * h->df_grid);
-    sbd_ns[i] = sm[(size_t)2 * i];
-    mbd_ns[i] = sm[(size_t)2 * i + 1];
-  }
-  FRBX_CK(h, cudaMemcpyAsync(b + o_sm, sm.data(), 16 * (size_t)n_bl, cudaMemcpyHostToDevice, st));
   const double f0_min = *std::min_element(h->f0.begin(), h->f0.end());
-  FRBX_CK(h, frbx::launch_cal_channels((const double2 *)(b + o_xs), h->d_wrot, n_bl, N, h->J, h->f_bw, h->d_f0,
-                                       f0_min, (const double *)(b + o_sm), (double *)(b + o_d),
-                                       (double *)(b + o_p), st, &h->launches));
-  FRBX_CK(h, cudaMemcpyAsync(delay_ns, b + o_d, 8 * (size_t)n_bl * N, cudaMemcpyDeviceToHost, st));
-  FRBX_CK(h, cudaMemcpyAsync(phase_rad, b + o_p, 8 * (size_t)n_bl * N, cudaMemcpyDeviceToHost, st));
+  double *d_out = (double *)(b + o_out);
+  FRBX_CK(h, frbx::launch_cal_channels((const double2 *)(b + o_xs), h->d_wrot, a.out, n_bl, N, h->J, h->Ls, h->Lm,
+                                       h->f_bw, h->df_grid, h->d_f0, f0_min, d_out, d_out + n_bl, d_out + 2 * n_bl,
+                                       d_out + (size_t)n_bl * (2 + N), st, &h->launches));
+  std::vector<double> out(n_out);
+  FRBX_CK(h, cudaMemcpyAsync(out.data(), d_out, 8 * n_out, cudaMemcpyDeviceToHost, st));
   FRBX_CK(h, cudaStreamSynchronize(st));
+  const double *o = out.data();
+  std::copy(o, o + n_bl, sbd_ns);
+  std::copy(o + n_bl, o + 2 * n_bl, mbd_ns);
+  std::copy(o + 2 * n_bl, o + (size_t)n_bl * (2 + N), delay_ns);
+  std::copy(o + (size_t)n_bl * (2 + N), o + n_out, phase_rad);
   return FRBX_OK;
 }
 
