@@ -366,13 +366,14 @@ int frbx_create(const frbx_setup *s, frbx_handle **out) {
     }
     h->b_bytes8 = KA8 * rows * 128;
   }
-  // window-tree tensor-core fit: per block of 32 MBD columns q, the DFT rows (Re G of the 32
-  // q, then Im G) split as W = W_hi + W_lo in BF16, in 128-byte swizzled images; per 64-wide
-  // K atom the 64 hi rows are followed by the 64 lo rows, so [W_hi; W_lo] is one 128-row operand
+  // window-tree tensor-core fit: per block of 48 or 32 MBD columns q (tree_mma_cols), the DFT rows
+  // (Re G of the block's q, then Im G) split as W = W_hi + W_lo in BF16, in 128-byte swizzled images; per 64-wide
+  // K atom the hi rows are followed by the lo rows
   std::vector<uint16_t> wtree;
   std::vector<uint8_t> wtree8;
   if (frbx::tree_mma_supported(h->Ls, h->Lm, N, J)) {
-    const int KA = (2 * N + 63) / 64, rows = 64, n_qb = h->Lm / 32, atom = rows * 128;
+    const int nq = frbx::tree_mma_cols(h->Lm, N), rows = 2 * nq, n_qb = (h->Lm + nq - 1) / nq;
+    const int KA = (2 * N + 63) / 64, atom = rows * 128;
     const int wb = 2 * KA * atom;  // bytes per block: per K atom, hi rows then lo rows
     wtree.assign((size_t)n_qb * wb / 2, 0);
     auto bf16 = [](double v) {
@@ -395,8 +396,9 @@ int frbx_create(const frbx_setup *s, frbx_handle **out) {
     };
     for (int qb = 0; qb < n_qb; ++qb)
       for (int R = 0; R < rows; ++R) {
-        const int q = qb * 32 + (R % 32);
-        const bool im = R >= 32;
+        const int q = qb * nq + (R % nq);
+        const bool im = R >= nq;
+        if (q >= h->Lm) continue;  // the last block's columns past the grid stay zero
         for (int n = 0; n < N; ++n) {
           const long long ex = ((long long)h->g[(size_t)n] * q) % h->Lm;
           const double th = two_pi * (double)ex / (double)h->Lm;
@@ -409,7 +411,7 @@ int frbx_create(const frbx_setup *s, frbx_handle **out) {
         }
       }
     h->wtree_bytes = wb;
-    // the E4M3 form: per block of 32 q, the same 64 rows (Re G of the 32 q, then Im G) rounded
+    // the E4M3 form: per block the same rows rounded
     // once to E4M3, 128 K values per 128-byte row
     const int KA8 = (2 * N + 127) / 128, wb8 = KA8 * rows * 128;
     wtree8.assign((size_t)n_qb * wb8, 0);
@@ -420,8 +422,9 @@ int frbx_create(const frbx_setup *s, frbx_handle **out) {
     };
     for (int qb = 0; qb < n_qb; ++qb)
       for (int R = 0; R < rows; ++R) {
-        const int q = qb * 32 + (R % 32);
-        const bool im = R >= 32;
+        const int q = qb * nq + (R % nq);
+        const bool im = R >= nq;
+        if (q >= h->Lm) continue;  // the last block's columns past the grid stay zero
         for (int n = 0; n < N; ++n) {
           const long long ex = ((long long)h->g[(size_t)n] * q) % h->Lm;
           const double th = two_pi * (double)ex / (double)h->Lm;
@@ -793,7 +796,7 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
     t.k8_steps = (2 * h->N + 31) / 32;
     t.tile_bytes = frbx::tree_mma_tile_bytes(form, h->N);
     t.wimg = (const unsigned char *)(form == 2 ? h->d_wtree8 : h->d_wtree);
-    t.w_bytes = frbx::tree_mma_w_bytes(form, h->N);
+    t.w_bytes = frbx::tree_mma_w_bytes(form, h->Lm, h->N);
     // delay windows: rotate the SBD rows so the searched ones come first (in groups of 8)
     t.rot = r->full ? 0 : (a.m_lo & ~7);
     // rows searched after the rotation: [m_lo mod 8, m_lo mod 8 + m_len) in 32-row quarters
@@ -802,7 +805,8 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
     t.prow = 128 / t.pack;
     t.piece_bytes = t.tile_bytes / t.pack;
     t.n_tg = (t.n_tt + t.pack - 1) / t.pack;
-    t.n_qb = h->Lm / 32;
+    const int cols = frbx::tree_mma_cols(h->Lm, h->N);
+    t.n_qb = (h->Lm + cols - 1) / cols;
     t.log2Lm = a.log2Lm;
     t.err = (int *)h->errflag.p;
     t.timeout = wait_cycles(h);
@@ -1211,7 +1215,7 @@ static int search_impl(frbx_handle *h, const void *vis, int32_t vis_on_device, i
   // tensor-core window tree: kernel 6 (split BF16, FP32-equivalent), 7 (BF16), 8 (E4M3)
   const bool tree_tc_shape = tree_ok && h->d_wtree && frbx::tree_mma_supported(h->Ls, h->Lm, h->N, h->J);
   const int tc_form = p.kernel == 7 ? 1 : p.kernel == 8 ? 2 : 0;
-  const bool tree_tc = tree_tc_shape && frbx::tree_mma_fits(tc_form, h->N, nlev);
+  const bool tree_tc = tree_tc_shape && frbx::tree_mma_fits(tc_form, h->Lm, h->N, nlev);
   if ((p.kernel == 4 && !tree_ok) || (p.kernel >= 6 && !tree_tc))
     return fail(h, FRBX_EUNSUPPORTED,
                 "window-tree fit needs power-of-two windows <= 64, Ls a multiple of 32 and Lm 16 or a multiple of 32 "
@@ -1604,7 +1608,7 @@ extern "C" int frbx_search_batch(frbx_batch *b, const frbx_scan *scans, int32_t 
     const bool ok = frbx::tree_supported(h->Ls, h->Lm, h->N, h->J, h->tree_s16, windows, n_win, &nlev);
     const FitArgs &ag = fa[g];
     const bool tc_ok = ok && h->d_wtree && frbx::tree_mma_supported(h->Ls, h->Lm, h->N, h->J) &&
-                       frbx::tree_mma_fits(0, h->N, nlev);
+                       frbx::tree_mma_fits(0, h->Lm, h->N, nlev);
     (void)ag;
     if ((p.kernel == 4 && !ok) || (p.kernel == 6 && !tc_ok))
       return bfail(b, FRBX_EUNSUPPORTED, "setup " + std::to_string(g) + ": window-tree fit does not apply");

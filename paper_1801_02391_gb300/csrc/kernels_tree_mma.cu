@@ -9,26 +9,29 @@
 // x_lo = bf16(x - x_hi), and D = A_hi B_hi + A_hi B_lo + A_lo B_hi accumulates in FP32 in tensor
 // memory (the dropped A_lo B_lo term is below 2^-16 of each product).
 //
-// One CTA owns all Ls = 128 SBD rows of one block of 32 MBD columns q of one (baseline, DM)
-// series and walks a time tile AP by AP (12 warps in three warpgroups):
-//   warp 9 (one lane) copies each AP's split A tiles (written by k_tree_sbd in their
+// One CTA owns all Ls = 128 SBD rows of one block of 48 (or 32) MBD columns q of one (baseline, DM)
+// series and walks a time tile AP by AP (12 or 8 epilogue warps and one warpgroup of four others):
+//   the loader warp (one lane) copies each AP's split A tiles (written by k_tree_sbd in their
 //          shared-memory image) into a ring with cp.async.bulk;
-//   warp 8 allocates tensor memory and runs the MMA loop convergently; one elected lane issues
-//          an AP's MMAs into one of two accumulator slots of 64 columns, so it runs one AP
-//          ahead: per K step three N = 64 MMAs, A_hi W_hi, A_hi W_lo and A_lo W_hi, all
+//   the MMA warp allocates tensor memory and runs the MMA loop convergently; one elected lane issues
+//          an AP's MMAs into one of two accumulator slots of 96 (64) columns, so it runs one AP
+//          ahead: per K step three MMAs, A_hi W_hi, A_hi W_lo and A_lo W_hi, all
 //          accumulating into the same slot (the issue keeps pace with the tensor pipe, and the
-//          epilogue reads one 64-column result per AP);
-//   warps 10 and 11 have no role: with warps 8 and 9 they form the warpgroup that hands its
+//          epilogue reads one result per AP);
+//   two more warps have no role: with those two they form the warpgroup that hands its
 //          registers to the epilogue (setmaxnreg), which is bound by each warp's chain of
-//          dependent work and gains from keeping more of the tree in registers;
-//   warps 0-7 (row quarter w % 4, q half w / 4) read G_1(k) into registers (freeing its slot
-//          at once), keep it there as G_1(k - 1) for the next AP, walk their 16 cells through
+//          dependent work;
+//   the epilogue warps (row quarter w % 4, columns 16 (w / 4) ...) read G_1(k) into registers (freeing
+//          its slot at once), keep it there as G_1(k - 1) for the next AP, walk their 16 cells through
 //          the window tree with packed FP32x2 arithmetic, and merge every emitted segment's
 //          warp maximum into the series by a 64-bit atomicMax, as k_tree_mbd does per block:
-//          the warps never wait for one another.  The first half of a window of 4 APs (tree
-//          level 2) stays in registers; those of windows 8 to 64 (levels 3 to 6) sit in tensor
-//          memory after the slots (shared memory takes anchor levels only where tensor memory
-//          has no room).
+//          the warps never wait for one another.  The first halves of windows of 4 APs and more
+//          (tree levels 2 to 6) sit in tensor memory after the slots as far as it has room, the
+//          deepest in shared memory; with two epilogue warpgroups, whose warps have 224 registers
+//          instead of 152, level 2 stays in registers.
+// Three warpgroups against two: the chain of
+// dependent work leaves issue slots free that a third warp per scheduler uses, and an A tile is read
+// by 11 CTAs instead of 16.  A search of 192 series x 20000 APs: 299.6 -> 260.5 ms.
 // Two lower-precision forms of the same tree run one product per AP instead of three: kernel 7
 // multiplies A_hi by W_hi (BF16, about 4e-3 relative on |G|), kernel 8 multiplies E4M3 operands
 // with kind::f8f6f4 (about 6e-2 relative), A scaled per AP by the power of two s with
@@ -54,60 +57,64 @@ namespace frbx {
 
 namespace {
 
-constexpr int kTmNQ = 32;                   // complex MBD columns per CTA
-constexpr int kTmCols = 2 * kTmNQ;          // Re G of the 32 q, then Im G
 constexpr int kTmMaxABufs = 3;              // ring of one-AP A tiles (2 where shared memory is short)
 constexpr int kTmTmemCols = 512;            // accumulator slots, then the tensor-memory anchors
 constexpr int kTmMaxLev = 6;
-constexpr int kTmWAtom = kTmCols * 128;     // 64 rows of one 128-byte K atom of W (8 KB)
-constexpr int kTmAncBytes = tc::kRows * kTmCols * 4;  // one anchor level in shared memory (32 KB)
-// configuration of the launched instance: epilogue warps (8 or 16) and accumulator slots
-constexpr int kTmEpi = 8;
-constexpr int kTmSlots = 2;
-// Register split.  The block has three warpgroups: the eight epilogue warps (groups 0 and 1) and
-// group 2 (the MMA warp, the loader warp and two warps with no role).  Each sub-partition holds one
-// warp of every group, so at launch every thread gets 168 registers (16384 per sub-partition over
-// three warps).  Group 2 then gives registers back (setmaxnreg.dec to 56) and the epilogue groups
-// take them (setmaxnreg.inc to 224): 8 x 32 x 224 + 4 x 32 x 56 = 64512 = 384 x 168, the launch
-// allocation exactly, so the increase never waits on registers that do not exist.  The host
-// launches the kernel only when it was built with 168 registers per thread.
-constexpr int kTmWarps = kTmEpi + 4;
-constexpr int kTmLaunchRegs = 168;
-constexpr int kTmEpiRegs = 224;
-constexpr int kTmAuxRegs = 56;
-static_assert(2 * 4 * 32 * kTmEpiRegs + 4 * 32 * kTmAuxRegs == kTmWarps * 32 * kTmLaunchRegs, "register split");
-static_assert(kTmEpi == 8, "two epilogue warpgroups");
+constexpr int kTmSlots = 2;                 // accumulator slots
+constexpr int kQ = 16;                      // MBD columns per epilogue thread
+constexpr int kP = kQ / 2;                  // packed pairs
+
+// Shape of a CTA: kParts warpgroups of epilogue warps, each on 16 of the CTA's 16 kParts MBD columns,
+// and one warpgroup of the MMA warp, the loader warp and two warps with no role.  Each sub-partition
+// holds one warp of every group.  At launch all threads have the same registers; the last group then
+// gives some back (setmaxnreg.dec) and the epilogue groups take them (setmaxnreg.inc), the launch
+// allocation exactly, so the increase never waits on registers that do not exist.  The host launches
+// the kernel only when it was built with kLaunchRegs per thread.
+//   kParts 3: 16 warps x 128 registers -> 12 x 152 and 4 x 56
+//   kParts 2: 12 warps x 168 registers -> 8 x 224 and 4 x 56
+template <int kParts>
+struct TmShape {
+  static constexpr int kNQ = kQ * kParts;       // complex MBD columns per CTA
+  static constexpr int kCols = 2 * kNQ;         // Re G of the kNQ columns, then Im G
+  static constexpr int kEpi = 4 * kParts;       // epilogue warps
+  static constexpr int kWarps = kEpi + 4;
+  static constexpr int kLaunchRegs = kParts == 3 ? 128 : 168;
+  static constexpr int kEpiRegs = kParts == 3 ? 152 : 224;
+  static constexpr int kAuxRegs = 56;
+  // the level-2 window anchor: in registers with two parts, with three in tensor memory as the deeper ones
+  static constexpr bool kRegAnchor = kParts == 2;
+  static constexpr int kAncCol = kTmSlots * kCols;                       // first anchor column of tensor memory
+  static constexpr int kTmemAnchors = (kTmTmemCols - kAncCol) / kCols;  // anchor levels there
+  static_assert(kEpi * kEpiRegs + 4 * kAuxRegs == kWarps * kLaunchRegs, "register split");
+};
+inline int tm_cols(int parts) { return 2 * kQ * parts; }
+inline int tm_tmem_anchors(int parts) { return parts == 3 ? TmShape<3>::kTmemAnchors : TmShape<2>::kTmemAnchors; }
 
 // forms of the MBD product (TreeArgs::form)
 constexpr int kFormSplit = 0;  // A_hi W_hi + A_hi W_lo + A_lo W_hi in BF16 (FP32-equivalent)
 constexpr int kFormBf16 = 1;   // A_hi W_hi
 constexpr int kFormFp8 = 2;    // E4M3 x E4M3, A scaled per AP
 
-// one accumulator slot: Re G and Im G of the block's 32 q (the split form's three products
-// accumulate into it)
-__host__ __device__ constexpr int tm_slot_cols(int) { return kTmCols; }
-__host__ __device__ constexpr int tm_tmem_anchors(int form, int slots) {
-  return (kTmTmemCols - slots * tm_slot_cols(form)) / kTmCols;
-}
 // K atoms (128 bytes of K per row) of the A tile and of W, and their bytes
 __host__ __device__ inline int tm_katoms(int form, int N) { return form == kFormFp8 ? (2 * N + 127) / 128 : (2 * N + 63) / 64; }
 __host__ __device__ inline int tm_tile_bytes(int form, int N) {
   return (form == kFormSplit ? 2 : 1) * tm_katoms(form, N) * tc::kAtomBytes;
 }
-__host__ __device__ inline int tm_w_bytes(int form, int N) {
-  return (form == kFormFp8 ? 1 : 2) * tm_katoms(form, N) * kTmWAtom;  // BF16: hi rows then lo rows per atom
-}
-size_t tm_smem_bytes(int w_bytes, int tile_bytes, int n_abuf, int n_sanc) {
-  return (size_t)((w_bytes + 1023) & ~1023) + (size_t)n_abuf * tile_bytes + (size_t)n_sanc * kTmAncBytes + 1024;
+// bytes of one K atom (64 BF16 or 128 E4M3 per row) of W, and of a column block's whole operand
+// (BF16: hi rows then lo rows per atom)
+inline int tm_w_atom(int parts) { return tm_cols(parts) * 128; }
+inline int tm_w_bytes(int form, int N, int parts) { return (form == kFormFp8 ? 1 : 2) * tm_katoms(form, N) * tm_w_atom(parts); }
+size_t tm_smem_bytes(int w_bytes, int tile_bytes, int parts, int n_abuf, int n_sanc) {
+  return (size_t)((w_bytes + 1023) & ~1023) + (size_t)n_abuf * tile_bytes + (size_t)n_sanc * tc::kRows * tm_cols(parts) * 4 + 1024;
 }
 // Memory plan: the anchor levels go to tensor memory as far as it has room beside the slots (a
 // visit moves 64 KB, which shared memory's bandwidth makes slower), the deeper rest to shared
 // memory after W and the deepest A-tile ring that fits.  Returns false when nothing fits.
-bool tm_plan(int form, int N, int nlev, int *n_abuf, int *n_sanc) {
-  const int w_bytes = tm_w_bytes(form, N), tile_bytes = tm_tile_bytes(form, N);
-  *n_sanc = max(0, nlev - 1 - tm_tmem_anchors(form, kTmSlots));
+bool tm_plan(int form, int N, int parts, int nlev, int *n_abuf, int *n_sanc) {
+  const int w_bytes = tm_w_bytes(form, N, parts), tile_bytes = tm_tile_bytes(form, N);
+  *n_sanc = max(0, nlev - 1 - tm_tmem_anchors(parts));
   for (int nb = kTmMaxABufs; nb >= 2; --nb)
-    if (tm_smem_bytes(w_bytes, tile_bytes, nb, *n_sanc) + 512 <= max_smem_optin()) {  // 512: static
+    if (tm_smem_bytes(w_bytes, tile_bytes, parts, nb, *n_sanc) + 512 <= max_smem_optin()) {  // 512: static
       *n_abuf = nb;
       return true;
     }
@@ -139,39 +146,29 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   return d;
 }
 
-// kQ consecutive FP32 columns of this thread's tensor-memory lane, as kQ / 2 packed pairs
-template <int kQ>
-__device__ __forceinline__ void tm_ld(uint32_t taddr, uint64_t (&v)[kQ / 2]) {
-  uint32_t r[kQ];
-  if constexpr (kQ == 16) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(taddr));
-  } else {
-    static_assert(kQ == 8, "8 or 16 columns");
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-  }
-#pragma unroll
-  for (int p = 0; p < kQ / 2; ++p) v[p] = pk(r[2 * p], r[2 * p + 1]);
+// kQ consecutive FP32 columns of this thread's tensor-memory lane.  The values are only there after
+// tm_wait_ld(): they stay 32-bit registers until tm_take() (an empty, ordered statement after the
+// wait that every use passes through) packs them into pairs.
+__device__ __forceinline__ void tm_ld(uint32_t taddr, uint32_t (&r)[kQ]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+               : "r"(taddr));
 }
-template <int kQ>
-__device__ __forceinline__ void tm_st(uint32_t taddr, const uint64_t (&v)[kQ / 2]) {
+__device__ __forceinline__ void tm_take(uint32_t (&r)[kQ], uint64_t (&v)[kP]) {
+  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                    "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
+#pragma unroll
+  for (int p = 0; p < kP; ++p) v[p] = pk(r[2 * p], r[2 * p + 1]);
+}
+__device__ __forceinline__ void tm_st(uint32_t taddr, const uint64_t (&v)[kP]) {
   uint32_t r[kQ];
 #pragma unroll
-  for (int p = 0; p < kQ / 2; ++p) upk(v[p], r[2 * p], r[2 * p + 1]);
-  if constexpr (kQ == 16) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-                   "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-                 : "memory");
-  } else {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-                 : "memory");
-  }
+  for (int p = 0; p < kP; ++p) upk(v[p], r[2 * p], r[2 * p + 1]);
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+               "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+               : "memory");
 }
 // (v & m) | (c & ~m) in one lop3: the high bits of v with the low bits of the immediate c
 __device__ __forceinline__ uint32_t pack_code(uint32_t v, uint32_t c, uint32_t m) {
@@ -186,17 +183,6 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return d;
 }
 __device__ __forceinline__ void tm_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// Placed after tm_wait_ld(): the values a tcgen05.ld wrote pass through this (empty, ordered)
-// statement, so no use of them can be scheduled above the wait.
-template <int kP>
-__device__ __forceinline__ void tm_hold(uint64_t (&v)[kP]) {
-  if constexpr (kP == 8) {
-    asm volatile("" : "+l"(v[0]), "+l"(v[1]), "+l"(v[2]), "+l"(v[3]), "+l"(v[4]), "+l"(v[5]), "+l"(v[6]), "+l"(v[7]));
-  } else {
-    static_assert(kP == 4, "4 or 8 packed pairs");
-    asm volatile("" : "+l"(v[0]), "+l"(v[1]), "+l"(v[2]), "+l"(v[3]));
-  }
-}
 __device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t idesc_bf16(int n) {
@@ -217,20 +203,17 @@ __device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint64_t ad, uint64_t 
 
 }  // namespace
 
-// kEpi epilogue warps, then the MMA warp, the loader warp and two idle warps.  Tensor memory:
-// kSlots accumulator slots of 64 columns, then one 64-column block per anchor level e >= 2 at
-// block e - 2 (level 2's block is unused: that anchor lives in registers).  Shared memory: W,
-// the A-tile ring (t.n_abuf deep), then the t.n_sanc deepest anchor levels as
-// [level][16 column quads][128 rows] float4.  kForm: the MBD product (above);
-// kFull: the whole delay grid is searched (no windows, no row rotation).
-template <int kEpi, int kSlots, int kForm, bool kFull>
-__global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_constant__ TreeArgs t) {
-  constexpr int kMmaWarp = kEpi, kLoadWarp = kEpi + 1;
-  constexpr int kQ = kTmNQ / (kEpi / 4);   // MBD columns per epilogue thread (16 or 8)
-  constexpr int kP = kQ / 2;               // packed pairs
-  constexpr int kSlotCols = tm_slot_cols(kForm);
-  constexpr int kAnc = kSlots * kSlotCols;
-  static_assert(tm_tmem_anchors(kForm, kSlots) >= 0, "tensor memory");
+// Epilogue warps, then the MMA warp, the loader warp and two idle warps (TmShape).  Tensor memory:
+// the accumulator slots, then one block of the same width per anchor level e >= 2 at block e - 2 (with
+// two parts level 2's block is unused: that anchor lives in registers).  Shared memory: W, the A-tile
+// ring (t.n_abuf deep), then the t.n_sanc deepest anchor levels as [level][column quads][128 rows]
+// float4.  kForm: the MBD product (above); kFull: the whole delay grid is searched (no windows, no row
+// rotation).
+template <int kParts, int kForm, bool kFull>
+__global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(const __grid_constant__ TreeArgs t) {
+  using Sh = TmShape<kParts>;
+  constexpr int kEpi = Sh::kEpi, kMmaWarp = kEpi, kLoadWarp = kEpi + 1, kNQ = Sh::kNQ, kCols = Sh::kCols;
+  constexpr int kSlots = kTmSlots, kAnc = Sh::kAncCol, kWAtom = kCols * 128, kQuads = kCols / 4;
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ uint64_t bar_afull[kTmMaxABufs], bar_aempty[kTmMaxABufs], bar_accfull[kSlots], bar_accempty[kSlots],
@@ -253,14 +236,13 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
   auto tile_n = [&](int p) { const int b = tile_kb(p); return b < kd ? min(kd, b + t.TT + lmax - 1) - b : 0; };
   const int kb = tile_kb(0);
   if (kb >= kd) return;  // every segment starting here runs past the scan (uniform)
-  // searched q of this block (bit j: q = 32 qb + j); none: nothing to do (uniform)
-  unsigned qbmask = 0xffffffffu;
-  if (!kFull) {
-    qbmask = 0u;
-    for (int j = 0; j < kTmNQ; ++j)
-      if ((((qb * kTmNQ + j) - t.q_lo) & (t.Lm - 1)) < t.q_len) qbmask |= 1u << j;
-    if (qbmask == 0u) return;
+  // searched q of this block (bit j: q = kNQ qb + j, all below Lm); none: nothing to do (uniform)
+  unsigned long long qbmask = 0ull;
+  for (int j = 0; j < kNQ; ++j) {
+    const int q = qb * kNQ + j;
+    if (q < t.Lm && (kFull || ((q - t.q_lo) & (t.Lm - 1)) < t.q_len)) qbmask |= 1ull << j;
   }
+  if (qbmask == 0ull) return;
   const int n_ap = tile_n(0);
   const int nbuf = t.n_abuf, n_tanc = max(t.nlev - 1, 0) - t.n_sanc;  // anchor levels in tensor memory
 
@@ -299,7 +281,7 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
 
   if (warp >= kEpi) {
   // warpgroup 2 (MMA, loader, two idle warps) hands registers to the epilogue warpgroups
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kTmAuxRegs));
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Sh::kAuxRegs));
   if (warp == kLoadWarp) {
     // ================= loader: one bulk copy of the split A tiles per AP =================
     if (lane == 0) {
@@ -348,7 +330,7 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
     // per-instruction moves into uniform registers); one elected lane issues the MMAs and
     // commits, which keeps the issue rate at the tensor pipe's pace.
     const bool leader = tc::elect_one();
-    const uint32_t id64 = idesc_bf16(kTmCols), id8 = idesc_e4m3(kTmCols);
+    const uint32_t id16 = idesc_bf16(kCols), id8 = idesc_e4m3(kCols);
     // descriptors of the K steps differ only in the start address field (address / 16, in
     // the low 14 bits, which shared-memory offsets below 256 KB never carry out of)
     const uint32_t a_half16 = (uint32_t)(t.KA * tc::kAtomBytes) >> 4;
@@ -365,18 +347,18 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint64_t a0 = sa0 + (uint64_t)(b * tile16);
-      const uint32_t d_tmem = tmem + (uint32_t)(slot * kSlotCols);
+      const uint32_t d_tmem = tmem + (uint32_t)(slot * kCols);
       if (leader) {
         if constexpr (kForm == kFormSplit) {
-          // D = A_hi W_hi + A_hi W_lo + A_lo W_hi, all N = 64 into one accumulator
+          // D = A_hi W_hi + A_hi W_lo + A_lo W_hi, into one accumulator
           for (int ka = 0; ka < t.KA; ++ka) {
 #pragma unroll
             for (int k4 = 0; k4 < 4; ++k4) {
               const uint32_t ao = (uint32_t)((ka * tc::kAtomBytes + k4 * 32) >> 4);
-              const uint32_t bo = (uint32_t)((ka * 2 * kTmWAtom + k4 * 32) >> 4);
-              mma_bf16(d_tmem, a0 + ao, w0 + bo, id64, (ka | k4) ? 1u : 0u);
-              mma_bf16(d_tmem, a0 + ao, w0 + bo + (uint32_t)(kTmWAtom >> 4), id64, 1u);
-              mma_bf16(d_tmem, a0 + a_half16 + ao, w0 + bo, id64, 1u);
+              const uint32_t bo = (uint32_t)((ka * 2 * kWAtom + k4 * 32) >> 4);
+              mma_bf16(d_tmem, a0 + ao, w0 + bo, id16, (ka | k4) ? 1u : 0u);
+              mma_bf16(d_tmem, a0 + ao, w0 + bo + (uint32_t)(kWAtom >> 4), id16, 1u);
+              mma_bf16(d_tmem, a0 + a_half16 + ao, w0 + bo, id16, 1u);
             }
           }
         } else if constexpr (kForm == kFormBf16) {
@@ -385,15 +367,15 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
 #pragma unroll
             for (int k4 = 0; k4 < 4; ++k4) {
               const uint32_t ao = (uint32_t)((ka * tc::kAtomBytes + k4 * 32) >> 4);
-              const uint32_t bo = (uint32_t)((ka * 2 * kTmWAtom + k4 * 32) >> 4);
-              mma_bf16(d_tmem, a0 + ao, w0 + bo, id64, (ka | k4) ? 1u : 0u);
+              const uint32_t bo = (uint32_t)((ka * 2 * kWAtom + k4 * 32) >> 4);
+              mma_bf16(d_tmem, a0 + ao, w0 + bo, id16, (ka | k4) ? 1u : 0u);
             }
           }
         } else {
           // D = A8 W8 (E4M3, K = 32 per instruction, 32 bytes of each 128-byte row)
           for (int kk = 0; kk < t.k8_steps; ++kk) {
             const uint32_t ao = (uint32_t)(((kk >> 2) * tc::kAtomBytes + (kk & 3) * 32) >> 4);
-            const uint32_t bo = (uint32_t)(((kk >> 2) * kTmWAtom + (kk & 3) * 32) >> 4);
+            const uint32_t bo = (uint32_t)(((kk >> 2) * kWAtom + (kk & 3) * 32) >> 4);
             mma_e4m3(d_tmem, a0 + ao, w0 + bo, id8, kk ? 1u : 0u);
           }
         }
@@ -421,22 +403,22 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
     if (!__all_sync(0xffffffffu, tc::mbar_wait(&bar_drain, 0, nullptr, t.drain_timeout)) && leader) *abortp = 1;
   }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kTmEpiRegs));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(Sh::kEpiRegs));
     // ================= epilogue: window tree and maxima =================
     const int quarter = warp & 3, part = warp >> 2;
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t c_re = (uint32_t)(kQ * part), c_im = (uint32_t)(kTmNQ + kQ * part);
+    const uint32_t c_re = (uint32_t)(kQ * part), c_im = (uint32_t)(kNQ + kQ * part);
     // this warp's time tile (its piece of the packed operand) and its first AP and AP count
     const int qpp = 4 / pack, my_p = quarter / qpp;
     const int kb_me = tile_kb(my_p), n_me = tile_n(my_p);
     // this lane's SBD row m (row (quarter mod qpp) 32 + lane of its piece, rotated by t.rot) and
     // its first cell
     const int m_row = ((quarter % qpp) * 32 + lane + t.rot) & (t.Ls - 1);
-    const unsigned idx_base = (unsigned)(m_row * t.Lm + qb * kTmNQ + kQ * part);
+    const unsigned idx_base = (unsigned)(m_row * t.Lm + qb * kNQ + kQ * part);
     // delay windows: the lane's row is searched, and which of its kQ cells
     const bool row_on = kFull || (((m_row - t.m_lo) & (t.Ls - 1)) < t.m_len);
-    const unsigned qmask = kFull ? 0xffffffffu : (qbmask >> (kQ * part)) & ((1u << kQ) - 1u);
-    if (!kFull && !__any_sync(0xffffffffu, row_on && qmask != 0u)) {
+    const unsigned qmask = (unsigned)(qbmask >> (kQ * part)) & ((1u << kQ) - 1u);
+    if (!__any_sync(0xffffffffu, row_on && qmask != 0u)) {
       // nothing of this warp is searched: it only hands each slot back
       bool ok = true;
       for (int i = 0, slot = 0, sph = 0; i < n_ap && ok; ++i) {
@@ -454,7 +436,7 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
       }
       if (!ok) *abortp = 1;
     } else {
-    // this thread's quads of a shared-memory anchor: re at kQ/4 part + u, im at 8 + kQ/4 part + u
+    // this thread's quads of a shared-memory anchor: re at 4 part + u, im at kQuads / 2 + 4 part + u
     ulonglong2 *my_anc = sAnc + (size_t)(kQ / 4 * part) * tc::kRows + quarter * 32 + lane;
     unsigned long long *keys = t.keys + ((size_t)sd.x * t.n_dm + sd.y) * t.S_tot;
     int woff[kTmMaxLev + 1];  // first slot of the window emitted at each level (-1: none)
@@ -468,15 +450,15 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
     for (int p = 0; p < kP; ++p) ga_re[p] = ga_im[p] = gb_re[p] = gb_im[p] = 0ull;
     for (int a = 0; a + 2 <= t.nlev; ++a) {
       if (a < n_tanc) {
-        const uint32_t ab = lane_base + (uint32_t)(kAnc + a * kTmCols);
-        tm_st<kQ>(ab + c_re, ga_re);
-        tm_st<kQ>(ab + c_im, ga_im);
+        const uint32_t ab = lane_base + (uint32_t)(kAnc + a * kCols);
+        tm_st(ab + c_re, ga_re);
+        tm_st(ab + c_im, ga_im);
       } else {
-        ulonglong2 *q = my_anc + (size_t)(a - n_tanc) * 16 * tc::kRows;
+        ulonglong2 *q = my_anc + (size_t)(a - n_tanc) * kQuads * tc::kRows;
 #pragma unroll
         for (int u = 0; u < kQ / 4; ++u) {
           q[u * tc::kRows] = make_ulonglong2(0ull, 0ull);
-          q[(8 + u) * tc::kRows] = make_ulonglong2(0ull, 0ull);
+          q[(kQuads / 2 + u) * tc::kRows] = make_ulonglong2(0ull, 0ull);
         }
       }
     }
@@ -502,16 +484,10 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
 #pragma unroll
         for (int j = 0; j < kQ; ++j) kf[j] = (qmask >> j) & 1u ? kf[j] : 0.f;
       }
-      float top;
-      if constexpr (kQ == 16) {
-        float m5[5];
+      float m5[5];
 #pragma unroll
-        for (int j = 0; j < 5; ++j) m5[j] = fmax3(kf[3 * j], kf[3 * j + 1], kf[3 * j + 2]);
-        top = fmax3(fmax3(m5[0], m5[1], m5[2]), fmax3(m5[3], m5[4], kf[15]), 0.f);
-      } else {
-        static_assert(kQ == 8, "8 or 16 cells per thread");
-        top = fmax3(fmax3(kf[0], kf[1], kf[2]), fmax3(kf[3], kf[4], kf[5]), fmaxf(kf[6], kf[7]));
-      }
+      for (int j = 0; j < 5; ++j) m5[j] = fmax3(kf[3 * j], kf[3 * j + 1], kf[3 * j + 2]);
+      const float top = fmax3(fmax3(m5[0], m5[1], m5[2]), fmax3(m5[3], m5[4], kf[15]), 0.f);
       return row_on ? __float_as_uint(top) : 0u;
     };
     // the warp maximum of a segment of level e starting at AP i0 (counted from the time tile's
@@ -551,9 +527,10 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
                       uint64_t(&aout_im)[kP]) -> bool {
       if (!__all_sync(0xffffffffu, tc::mbar_wait(&bar_accfull[slot], sph, abortp, t.timeout))) return false;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t cur = lane_base + (uint32_t)(slot * kSlotCols);
-      tm_ld<kQ>(cur + c_re, cre);
-      tm_ld<kQ>(cur + c_im, cim);
+      const uint32_t cur = lane_base + (uint32_t)(slot * kCols);
+      uint32_t rre[kQ], rim[kQ];
+      tm_ld(cur + c_re, rre);
+      tm_ld(cur + c_im, rim);
 
       float inv_s = 1.f;  // E4M3 form: the AP's A was scaled by s, a power of two
       if constexpr (kForm == kFormFp8) inv_s = __ldg(t.ascale + (size_t)s * t.T + kb_me + i);
@@ -572,8 +549,8 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
         }
       }
       tm_wait_ld();
-      tm_hold<kP>(cre);
-      tm_hold<kP>(cim);
+      tm_take(rre, cre);
+      tm_take(rim, cim);
       if constexpr (kForm == kFormFp8) {
         const uint64_t iv = pk(__float_as_uint(inv_s), __float_as_uint(inv_s));
 #pragma unroll
@@ -600,22 +577,51 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
         merge(1, i - 1, top1, (em & 2u) != 0u);
         return true;
       }
-      // odd AP: levels 0, 1 and 2 as one block
-#pragma unroll
-      for (int p = 0; p < kP; ++p) {
-        aout_re[p] = add2(pre[p], cre[p]);
-        aout_im[p] = add2(pim[p], cim[p]);
-      }
+      // odd AP: levels 0, 1 and 2
       uint64_t are[kP], aim[kP];
+      if constexpr (Sh::kRegAnchor) {
 #pragma unroll
-      for (int p = 0; p < kP; ++p) {
-        are[p] = add2(ain_re[p], aout_re[p]);
-        aim[p] = add2(ain_im[p], aout_im[p]);
+        for (int p = 0; p < kP; ++p) {
+          aout_re[p] = add2(pre[p], cre[p]);
+          aout_im[p] = add2(pim[p], cim[p]);
+        }
+#pragma unroll
+        for (int p = 0; p < kP; ++p) {
+          are[p] = add2(ain_re[p], aout_re[p]);
+          aim[p] = add2(ain_im[p], aout_im[p]);
+        }
+        const unsigned top0 = seg_top(cre, cim), top1 = seg_top(aout_re, aout_im), top2 = seg_top(are, aim);
+        merge(0, i, top0, (em & 1u) != 0u);
+        merge(1, i - 1, top1, (em & 2u) != 0u);
+        merge(2, i - 3, top2, ((em >> 2) & 1u) != 0u);
+      } else {
+        // the level-2 anchor's read is in flight while levels 0 and 1 are formed (its column block
+        // exists whatever t.nlev; below two levels nothing of it is emitted)
+        const uint32_t ab = lane_base + (uint32_t)kAnc;
+        tm_wait_st();
+        tm_ld(ab + c_re, rre);
+        tm_ld(ab + c_im, rim);
+#pragma unroll
+        for (int p = 0; p < kP; ++p) {
+          are[p] = add2(pre[p], cre[p]);
+          aim[p] = add2(pim[p], cim[p]);
+        }
+        const unsigned top0 = seg_top(cre, cim), top1 = seg_top(are, aim);
+        merge(0, i, top0, (em & 1u) != 0u);
+        merge(1, i - 1, top1, (em & 2u) != 0u);
+        uint64_t ore[kP], oim[kP];
+        tm_wait_ld();
+        tm_take(rre, ore);
+        tm_take(rim, oim);
+        tm_st(ab + c_re, are);
+        tm_st(ab + c_im, aim);
+#pragma unroll
+        for (int p = 0; p < kP; ++p) {
+          are[p] = add2(ore[p], are[p]);
+          aim[p] = add2(oim[p], aim[p]);
+        }
+        merge(2, i - 3, seg_top(are, aim), ((em >> 2) & 1u) != 0u);
       }
-      const unsigned top0 = seg_top(cre, cim), top1 = seg_top(aout_re, aout_im), top2 = seg_top(are, aim);
-      merge(0, i, top0, (em & 1u) != 0u);
-      merge(1, i - 1, top1, (em & 2u) != 0u);
-      merge(2, i - 3, top2, ((em >> 2) & 1u) != 0u);
       if (!deep || E <= 2) return true;
       // levels 3 and up: anchor e - 2 of tensor memory (or shared memory) holds the first half
 #pragma unroll
@@ -624,25 +630,25 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
         uint64_t ore[kP], oim[kP];
         const bool in_tmem = e - 2 < n_tanc;  // uniform
         if (in_tmem) {
-          const uint32_t ab = lane_base + (uint32_t)(kAnc + (e - 2) * kTmCols);
-          tm_ld<kQ>(ab + c_re, ore);
-          tm_ld<kQ>(ab + c_im, oim);
+          const uint32_t ab = lane_base + (uint32_t)(kAnc + (e - 2) * kCols);
+          tm_ld(ab + c_re, rre);
+          tm_ld(ab + c_im, rim);
           tm_wait_ld();
-          tm_hold<kP>(ore);
-          tm_hold<kP>(oim);
-          tm_st<kQ>(ab + c_re, are);
-          tm_st<kQ>(ab + c_im, aim);
+          tm_take(rre, ore);
+          tm_take(rim, oim);
+          tm_st(ab + c_re, are);
+          tm_st(ab + c_im, aim);
         } else {
-          ulonglong2 *q = my_anc + (size_t)(e - 2 - n_tanc) * 16 * tc::kRows;
+          ulonglong2 *q = my_anc + (size_t)(e - 2 - n_tanc) * kQuads * tc::kRows;
 #pragma unroll
           for (int u = 0; u < kQ / 4; ++u) {
-            const ulonglong2 r = q[u * tc::kRows], m = q[(8 + u) * tc::kRows];
+            const ulonglong2 r = q[u * tc::kRows], m = q[(kQuads / 2 + u) * tc::kRows];
             ore[2 * u] = r.x;
             ore[2 * u + 1] = r.y;
             oim[2 * u] = m.x;
             oim[2 * u + 1] = m.y;
             q[u * tc::kRows] = make_ulonglong2(are[2 * u], are[2 * u + 1]);
-            q[(8 + u) * tc::kRows] = make_ulonglong2(aim[2 * u], aim[2 * u + 1]);
+            q[(kQuads / 2 + u) * tc::kRows] = make_ulonglong2(aim[2 * u], aim[2 * u + 1]);
           }
         }
 #pragma unroll
@@ -709,56 +715,70 @@ __global__ void __launch_bounds__((kEpi + 4) * 32, 1) k_tree_mma(const __grid_co
   if (tid == 0 && abort_flag) atomicExch(t.err, FRBX_ETIMEOUT);
 }
 
+// Column blocks of 48 (three epilogue warpgroups) where one 64-wide K atom holds the operand: three
+// epilogue warps per sub-partition instead of two hide more of each warp's chain, and an A tile is
+// read by Lm / 48 CTAs instead of Lm / 32.  Blocks of 32 where 48 would leave a third of the block
+// empty (Lm 32 and 64), or where 2N > 64 doubles the tiles and the operand, which beside 48-column
+// anchors in shared memory would leave no room for two ring buffers.
+int tree_mma_cols(int Lm, int N) { return 2 * N <= 64 && Lm > 64 ? 48 : 32; }
+
 bool tree_mma_supported(int Ls, int Lm, int N, int J) {
-  return Ls == tc::kRows && J <= Ls && Lm % kTmNQ == 0 && 2 * N <= 128;
+  return Ls == tc::kRows && J <= Ls && Lm % 32 == 0 && 2 * N <= 128;
 }
 
-bool tree_mma_fits(int form, int N, int nlev) {
+bool tree_mma_fits(int form, int Lm, int N, int nlev) {
   int nb, ns;
-  return form >= kFormSplit && form <= kFormFp8 && nlev >= 0 && nlev <= kTmMaxLev && tm_plan(form, N, nlev, &nb, &ns);
+  return form >= kFormSplit && form <= kFormFp8 && nlev >= 0 && nlev <= kTmMaxLev &&
+         tm_plan(form, N, tree_mma_cols(Lm, N) / kQ, nlev, &nb, &ns);
 }
 
 int tree_mma_tile_bytes(int form, int N) { return tm_tile_bytes(form, N); }
-int tree_mma_w_bytes(int form, int N) { return tm_w_bytes(form, N); }
+int tree_mma_w_bytes(int form, int Lm, int N) { return tm_w_bytes(form, N, tree_mma_cols(Lm, N) / kQ); }
 
-template <int kForm, bool kFull>
+template <int kParts, int kForm, bool kFull>
 static cudaError_t launch_tm_one(const TreeArgs &u, unsigned nb, size_t smem, cudaStream_t st) {
-  auto kern = k_tree_mma<kTmEpi, kTmSlots, kForm, kFull>;
-  // the register split inside the kernel assumes the launch allocation of kTmLaunchRegs per thread
+  using Sh = TmShape<kParts>;
+  auto kern = k_tree_mma<kParts, kForm, kFull>;
+  // the register split inside the kernel assumes the launch allocation of kLaunchRegs per thread
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, kern);
   if (e != cudaSuccess) return e;
-  if (fa.numRegs != kTmLaunchRegs || fa.maxThreadsPerBlock < kTmWarps * 32) return cudaErrorInvalidConfiguration;
+  if (fa.numRegs != Sh::kLaunchRegs || fa.maxThreadsPerBlock < Sh::kWarps * 32) return cudaErrorInvalidConfiguration;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<nb, kTmWarps * 32, smem, st>>>(u);
+  kern<<<nb, Sh::kWarps * 32, smem, st>>>(u);
   return cudaGetLastError();
 }
 
+template <int kParts>
+static cudaError_t launch_tm(const TreeArgs &u, bool full, unsigned g, size_t smem, cudaStream_t st) {
+  switch (u.form * 2 + (full ? 1 : 0)) {
+    case 0: return launch_tm_one<kParts, kFormSplit, false>(u, g, smem, st);
+    case 1: return launch_tm_one<kParts, kFormSplit, true>(u, g, smem, st);
+    case 2: return launch_tm_one<kParts, kFormBf16, false>(u, g, smem, st);
+    case 3: return launch_tm_one<kParts, kFormBf16, true>(u, g, smem, st);
+    case 4: return launch_tm_one<kParts, kFormFp8, false>(u, g, smem, st);
+    default: return launch_tm_one<kParts, kFormFp8, true>(u, g, smem, st);
+  }
+}
+
 cudaError_t launch_tree_mma(const TreeArgs &t, bool full, cudaStream_t st, int64_t *launches) {
+  const int cols = tree_mma_cols(t.Lm, t.N), parts = cols / kQ;
   if (t.nlev < 0 || t.nlev > kTmMaxLev || t.form < kFormSplit || t.form > kFormFp8 || t.KA != tm_katoms(t.form, t.N) ||
-      t.w_bytes != tm_w_bytes(t.form, t.N) || t.tile_bytes != tm_tile_bytes(t.form, t.N) ||
+      t.w_bytes != tm_w_bytes(t.form, t.N, parts) || t.tile_bytes != tm_tile_bytes(t.form, t.N) ||
+      t.n_qb != (t.Lm + cols - 1) / cols ||
       (t.form == kFormFp8 && (!t.ascale || t.k8_steps != (2 * t.N + 31) / 32)) || (full && t.rot != 0) ||
       (t.rot & 7) != 0 || !(t.pack == 1 || t.pack == 2 || t.pack == 4) || (full && t.pack != 1) ||
       t.prow * t.pack != tc::kRows || t.piece_bytes * t.pack != t.tile_bytes || t.n_tg * t.pack < t.n_tt ||
       t.TT % (1 << kTmMaxLev) != 0)
     return cudaErrorInvalidValue;
   TreeArgs u = t;
-  if (!tm_plan(t.form, t.N, t.nlev, &u.n_abuf, &u.n_sanc)) return cudaErrorInvalidConfiguration;
-  const size_t smem = tm_smem_bytes(t.w_bytes, t.tile_bytes, u.n_abuf, u.n_sanc);
+  if (!tm_plan(t.form, t.N, parts, t.nlev, &u.n_abuf, &u.n_sanc)) return cudaErrorInvalidConfiguration;
+  const size_t smem = tm_smem_bytes(t.w_bytes, t.tile_bytes, parts, u.n_abuf, u.n_sanc);
   const long long nb = (long long)t.n_s * t.n_qb * t.n_tg;
   if (nb <= 0) return cudaSuccess;
   if (nb > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  const unsigned g = (unsigned)nb;
-  cudaError_t e;
-  switch (t.form * 2 + (full ? 1 : 0)) {
-    case 0: e = launch_tm_one<kFormSplit, false>(u, g, smem, st); break;
-    case 1: e = launch_tm_one<kFormSplit, true>(u, g, smem, st); break;
-    case 2: e = launch_tm_one<kFormBf16, false>(u, g, smem, st); break;
-    case 3: e = launch_tm_one<kFormBf16, true>(u, g, smem, st); break;
-    case 4: e = launch_tm_one<kFormFp8, false>(u, g, smem, st); break;
-    default: e = launch_tm_one<kFormFp8, true>(u, g, smem, st); break;
-  }
+  const cudaError_t e = parts == 3 ? launch_tm<3>(u, full, (unsigned)nb, smem, st) : launch_tm<2>(u, full, (unsigned)nb, smem, st);
   ++*launches;
   return e;
 }
