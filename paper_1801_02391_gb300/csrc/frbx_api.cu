@@ -237,6 +237,15 @@ int frbx_create(const frbx_setup *s, frbx_handle **out) {
   h->Ls = sg.Ls;
   h->Lm = sg.Lm;
   h->J1 = (J + 31) / 32;
+  // refinement: APs a point's sweep moves per unit of DM (Eq. 1 over t_ap), FP32 frequencies
+  std::vector<frbx::RefinePoint> pts((size_t)h->C);
+  const double inv_fref2 = 1.0 / (h->f_ref * h->f_ref);
+  for (int c = 0; c < h->C; ++c) {
+    const double f = h->f[(size_t)c];
+    const double ddm = (4.15e6 * (1.0 / (f * f) - inv_fref2)) / h->t_ap;
+    const double fj = ((double)(c % J) * s->f_bw_mhz) / (double)J, fm = h->f0[(size_t)(c / J)] - sg.fmin0;
+    pts[(size_t)c] = {ddm, (float)fj, (float)fm, (float)ddm, 0};
+  }
   // weight x calibration rotation exp(-i[2 pi (f_j - f_bw/2) dtau0_n + dphi0_n]) (Eq. 5)
   const double two_pi = 6.283185307179586476925286766559;
   std::vector<float2> wrot((size_t)h->C);
@@ -436,6 +445,7 @@ int frbx_create(const frbx_setup *s, frbx_handle **out) {
   cudaError_t e = cudaGetDevice(&h->device);
   if (e == cudaSuccess) e = upload(&h->d_f, h->f);
   if (e == cudaSuccess) e = upload(&h->d_f0, h->f0);
+  if (e == cudaSuccess) e = upload(&h->d_pt, pts);
   if (e == cudaSuccess) e = upload(&h->d_wrot, wrot);
   if (e == cudaSuccess) e = upload(&h->d_tw_s, tws);
   if (e == cudaSuccess) e = upload(&h->d_tw_m, twm);
@@ -465,7 +475,7 @@ int frbx_create(const frbx_setup *s, frbx_handle **out) {
 
 void frbx_destroy(frbx_handle *h) {
   if (!h) return;
-  void *ptrs[] = {h->d_f,      h->d_f0,     h->d_wrot, h->d_tw_s, h->d_tw_m,     h->d_g,
+  void *ptrs[] = {h->d_f,      h->d_f0,     h->d_pt,    h->d_wrot, h->d_tw_s, h->d_tw_m,     h->d_g,
                   h->d_sbd_tw, h->d_mbd_tw, h->d_slot, h->d_bimg, h->d_tree_tw, h->d_tree_slot, h->d_bimg8,
                   h->d_wtree,  h->d_wtree8};
   for (void *p : ptrs)
@@ -1361,11 +1371,11 @@ int refine_common(frbx_handle *h, const void *vis_dev, int32_t n_bl, int32_t T, 
   r->n_bl = n_bl;
   r->n_cand = n_cand;
   r->n_par = 2 + 3 * n_bl;
-  r->f = h->d_f;
+  r->pt = h->d_pt;
   r->f0 = h->d_f0;
   r->wrot = h->d_wrot;
   r->f0_min = *std::min_element(h->f0.begin(), h->f0.end());
-  r->inv_fref2 = 1.0 / (h->f_ref * h->f_ref);
+  r->f0_max = *std::max_element(h->f0.begin(), h->f0.end());
   r->f_bw = h->f_bw;
   r->t_ap = h->t_ap;
   r->params = params_dev;

@@ -112,13 +112,18 @@ cudaError_t launch_fit_mma(const FitArgs &a, const MmaArgs &mm, int n_bl, bool l
                            int64_t *launches);
 
 // kernels_refine.cu: coherent power of continuous (DM, t0, tau_s, tau_m, rho) and its adjoint
+struct RefinePoint {
+  double ddm;              // du/dDM (APs per pc cm^-3)
+  float fj, fm, df;        // f_j, f0_n - min f0 (MHz) and du/dDM in FP32
+  int pad;
+};
 struct RefineArgs {
   const float2 *vis;       // [n_bl][T][C]
   int T, C, J, n_bl, n_cand, n_par;
-  const double *f;         // [C] point frequencies
+  const RefinePoint *pt;   // [C]
   const double *f0;        // [N] channel edges
   const float2 *wrot;      // [C]
-  double f0_min, inv_fref2, f_bw, t_ap;
+  double f0_min, f0_max, f_bw, t_ap;
   const double *params;    // [n_cand][n_par]
   const int *width;        // [n_cand]
   float *g;                // [n_cand][n_bl][2]
@@ -271,6 +276,7 @@ struct frbx_handle {
   double stage_ms[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
   // constant device tables
   double *d_f = nullptr, *d_f0 = nullptr;
+  frbx::RefinePoint *d_pt = nullptr;  // refinement: constants of every point
   float2 *d_wrot = nullptr, *d_tw_s = nullptr, *d_tw_m = nullptr;
   float2 *d_sbd_tw = nullptr, *d_mbd_tw = nullptr;
   float2 *d_tree_tw = nullptr;  // [16 s16][Lm/32][2] MBD twiddles of the window-tree fit

@@ -4,12 +4,29 @@
 //   u(n,j)   = t0 + 4.15e6 DM (f^-2 - f_ref^-2) / t_ap                  (FP64)
 //   X(i)     = sum_{m=-1..2} w_m(phi) S(n, j, k + m),  k + phi = u + i  (cubic Catmull-Rom)
 //   Phi      = 2 pi [ (f_j tau_s + (f0_n - f0_min) tau_m) 1e-3 + f0_n rho t_ap (u + i) 1e-6 ]
-//              (argument formed and reduced modulo one cycle in FP64, sine / cosine in FP32)
+//              (argument reduced modulo one cycle exactly, sine / cosine in FP32)
 //   G_b      = sum_{n, j>=1} c(n, j) sum_{i<l} X(i) exp(-i Phi),   P = sum_b |G_b|^2
 //
 // One CTA per (candidate, baseline); the adjoint accumulates dG_b/dtheta with the same walk
 // and contracts it with 2 conj(G_b) dL/dP.  Samples whose taps would leave the cube count as
 // zero and raise the candidate's status flag.
+//
+// FP64 (2 operations per cycle and SM against 128 in FP32) is what bounds this walk, and all of it ends
+// in values rounded to FP32: the tap position, the reduced phase, the factor of the rate's gradient.  So
+// FP64 is left to the position of each point, and the rounded results of a sample are found
+// another way, to the bit:
+//  * the tap position is the fraction of u for every sample, unless the rounding of u + i could show in
+//    FP32 (then sample by sample), so the weights are formed once per point and the taps slide;
+//  * the phase in cycles is kept as a 64-bit fixed-point fraction, whose wrap-around is the reduction
+//    modulo one cycle.  It is within `slack` of what the FP64 expression gives: unless a point where the
+//    rounding to FP32 changes is that near (about one sample in 10^4), its rounded value is the
+//    expression's; otherwise the expression is evaluated;
+//  * f0_n t_ap (u + i) is a sum of two floats, rounded under the same condition.
+// What a point contributes (du/dDM, its FP32 frequencies) is a table of the handle.  Forward and backward
+// of 200 candidates x 15 baselines x 2048 points, windows of 1 to 16 APs: 3.15 -> 0.77 ms, the same bits
+// (two baselines per CTA, to share their points' FP64: 0.85 ms, the CTAs of the longest windows end late).
+#include <climits>
+
 #include "frbx_internal.h"
 
 namespace frbx {
@@ -17,26 +34,11 @@ namespace frbx {
 namespace {
 
 constexpr int kRefThreads = 256;
+constexpr int kRefWarps = kRefThreads / 32;
+constexpr int kRefAhead = 4;       // samples whose taps are loaded together
 
 __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-
-struct PointConst {
-  double f, fj, f0n, fmbd, ddm;  // frequencies (MHz) and du/dDM (APs per pc cm^-3)
-  float2 wrot;
-};
-
-__device__ __forceinline__ PointConst point_const(const RefineArgs &r, int c) {
-  PointConst p;
-  const int n = c / r.J, j = c - n * r.J;
-  p.f = r.f[c];
-  p.fj = __ddiv_rn(__dmul_rn((double)j, r.f_bw), (double)r.J);
-  p.f0n = r.f0[n];
-  p.fmbd = p.f0n - r.f0_min;
-  p.ddm = __ddiv_rn(__dmul_rn(4.15e6, __dsub_rn(__ddiv_rn(1.0, __dmul_rn(p.f, p.f)), r.inv_fref2)), r.t_ap);
-  p.wrot = r.wrot[c];
-  return p;
 }
 
 __device__ __forceinline__ void cr_weights(float t, float w[4], float dw[4]) {
@@ -51,80 +53,262 @@ __device__ __forceinline__ void cr_weights(float t, float w[4], float dw[4]) {
   dw[3] = 0.5f * (3.f * t2 - 2.f * t);
 }
 
-// exp(-2 pi i cycles), the argument reduced modulo one in FP64 first
-__device__ __forceinline__ float2 phasor(double cycles) {
-  const double red = cycles - floor(cycles);
+constexpr double kTwo64 = 18446744073709551616.0;
+
+// What depends on opaque(v) is not computed ahead of where that stands.
+__device__ __forceinline__ double opaque(double v) {
+  asm volatile("" : "+d"(v));
+  return v;
+}
+
+// exact sum of two floats: a + b = s + e (Knuth's two-sum)
+__device__ __forceinline__ float two_sum(float a, float b, float &e) {
+  const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
+  return s;
+}
+
+// cycles modulo one in units of 2^-64 (two's complement)
+__device__ __forceinline__ unsigned long long cycle_fraction(double cycles) {
+  return (unsigned long long)__double2ll_rn((cycles - rint(cycles)) * kTwo64);
+}
+
+// A fraction of 2^-64 units rounded to FP32 (nearest, ties to even), valid when every value within slack
+// of it rounds alike: slack8 = slack / 2^8 rounded up, zmax = the most leading zeros at which the
+// interval still fits the bits below the rounding point.  False for fractions within reach of 0 or 1.
+__device__ __forceinline__ bool round_fraction(unsigned long long fr, unsigned slack8, int zmax, float &out) {
+  const unsigned hi = (unsigned)(fr >> 32), lo = (unsigned)fr;
+  const int z = __clz((int)hi);
+  const unsigned mh = __funnelshift_l(lo, hi, z), ml = lo << (z & 31);  // normalised: bit 31 of mh set
+  // the 40 bits below the 24 that stay, as their upper 32, against the half
+  const int off = (int)(__funnelshift_l(ml, mh, 24) ^ 0x80000000u);
+  out = __uint2float_rn(mh | (ml != 0u ? 1u : 0u)) * __int_as_float((127 - 32 - z) << 23);
+  return z <= zmax && hi != 0xffffffffu && (unsigned)abs(off) > (slack8 << (z & 31)) + 1u;
+}
+__device__ __forceinline__ int round_zmax(unsigned slack8) { return min(20, __clz((int)slack8) - 2); }
+
+// [0, 1) in units of 2^-64, truncated
+__device__ __forceinline__ unsigned long long unit_fraction(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int sh = (int)(b >> 52) - 1011;  // exponent 1022 (v in [0.5, 1)): 11 left
+  const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+  return sh >= 0 ? m << (sh & 63) : sh > -64 ? m >> (-sh) : 0ull;
+}
+
+// exp(-2 pi i red), red in [0, 1]
+__device__ __forceinline__ float2 phasor(float red) {
   float s, c;
-  sincospif(2.f * (float)red, &s, &c);
+  sincospif(2.f * red, &s, &c);
   return make_float2(c, -s);
 }
 
+// Phase of a channel of one baseline: offset and rate per AP in units of 2^-64 cycles, the rate's whole
+// cycles, and dPhi/du
+struct ChanPhase {
+  unsigned long long offset, rate;
+  long long whole;
+  float arate;
+};
+// A baseline: phase step per point (units of 2^-64 cycles) and the interval of round_fraction
+struct BlPhase {
+  unsigned long long step;
+  unsigned slack8;
+  int zmax;
+};
+
+// Sums v[] over the CTA; the result of value k is in out[k] after the closing barrier.
 template <int NV>
-__device__ __forceinline__ void block_sum(float (&v)[NV], float *red) {
+__device__ __forceinline__ void block_sum(const float (&v)[NV], float *red, float *out) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-  for (int k = 0; k < NV; ++k)
+  for (int k = 0; k < NV; ++k) {
+    float s = v[k];
 #pragma unroll
-    for (int off = 16; off; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < NV; ++k) red[k * 32 + warp] = v[k];
+    for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) red[k * kRefWarps + warp] = s;
+  }
   __syncthreads();
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      float s = 0.f;
-      for (int w = 0; w < nw; ++w) s += red[k * 32 + w];
-      v[k] = s;
+  for (int k = threadIdx.x; k < NV; k += kRefThreads) {
+    float s = 0.f;
+    for (int w = 0; w < kRefWarps; ++w) s += red[k * kRefWarps + w];
+    out[k] = s;
+  }
+  __syncthreads();
+}
+
+// The walk of one CTA: kVals sums (2 forward, 10 adjoint), in sums[].
+template <bool kAdjoint>
+__device__ __forceinline__ void refine_walk(const RefineArgs &r, int cand, int b, float *sums, bool &edge) {
+  constexpr int kVals = kAdjoint ? 10 : 2;
+  __shared__ ChanPhase s_ph[kMaxChan];
+  __shared__ BlPhase s_bl;
+  __shared__ float2 s_f0[kMaxChan];
+  __shared__ float red[kVals * kRefWarps];
+  const double *th = r.params + (size_t)cand * r.n_par;
+  const double dm = th[0], t0 = th[1], tau_s = th[2 + 3 * b], tau_m = th[3 + 3 * b], rho = th[4 + 3 * b];
+  const int N = r.C / r.J, l = r.width[cand];
+  for (int n = threadIdx.x; n < N; n += kRefThreads) {
+    const double f0n = r.f0[n], rate = f0n * rho * r.t_ap * 1e-6, whole = rint(rate);
+    s_ph[n] = {cycle_fraction((f0n - r.f0_min) * tau_m * 1e-3), cycle_fraction(rate), __double2ll_rn(whole),
+               (float)(6.283185307179586 * f0n * rho * r.t_ap * 1e-6)};
+  }
+  if (threadIdx.x == 0) {
+    // Terms of the phase at their largest, x <= T: each of the few roundings of the FP64 expression and of
+    // the fixed-point terms is below 2^-52 of them, and 2^-49 of their sum bounds all (the fixed-point
+    // rate's own unit, T times over, comes on top).  Too large (or not a number): no fraction passes
+    // round_fraction, every phase is evaluated.
+    const double big = (fabs(r.f_bw * tau_s) + fabs((r.f0_max - r.f0_min) * tau_m)) * 1e-3 +
+                       fabs(r.f0_max * rho * r.t_ap * 1e-6) * (r.T + 1.0);
+    // in units of 2^-56: 2^(64 - 49 - 8) = 128
+    const unsigned slack8 = big < 1e6 ? __double2uint_ru(big * 128.0) + 256u + (unsigned)(r.T >> 7) : 0xffffffffu;
+    s_bl = {cycle_fraction(r.f_bw / (double)r.J * tau_s * 1e-3), slack8, round_zmax(slack8)};
+  }
+  if (kAdjoint)
+    for (int n = threadIdx.x; n < N; n += kRefThreads) {
+      const double v = r.f0[n] * r.t_ap;
+      const float h = (float)v;
+      s_f0[n] = make_float2(h, (float)(v - (double)h));
     }
+  __syncthreads();
+  const double inv_j = 1.0 / (double)r.J;  // J is a power of two: exact
+  const float2 *const vb = r.vis + (size_t)b * r.T * r.C;
+  float ac[kVals];
+#pragma unroll
+  for (int k = 0; k < kVals; ++k) ac[k] = 0.f;
+  for (int c = threadIdx.x; c < r.C; c += kRefThreads) {
+    const float2 wr = r.wrot[c];
+    if (wr.x == 0.f && wr.y == 0.f) continue;  // j = 0 or flagged
+    const int n = c / r.J, j = c - n * r.J;
+    const RefinePoint pt = r.pt[c];
+    const double u = t0 + dm * pt.ddm;
+    // integer part and fraction of u (saturates; 0 for NaN, which no tap test passes below)
+    int k0 = __double2int_rd(u);
+    double fr = u - (double)k0;
+    if (fr >= 1.0) {  // u just below an integer that u + i rounds to
+      ++k0;
+      fr = 0.0;
+    }
+    const unsigned long long fr64 = unit_fraction(fr);
+    // |u + i| < 2^e is rounded by 2^(e - 54) at most: 2^(e + 2) units of 2^-56, here eight times that
+    const bool small = k0 > -(1 << 20) && k0 < (1 << 20) && l < (1 << 20);
+    const unsigned dw8 = small ? 32u << (32 - __clz(abs(k0) + l + 1)) : 0xffffffffu;
+    float frf;
+    const bool steady = round_fraction(fr64, dw8, round_zmax(dw8), frf);
+    float w[4], dw[4];
+    cr_weights(frf, w, dw);
+    const float f0h = s_f0[n].x, f0l = s_f0[n].y;  // f0_n t_ap
+    float bh = 0.f, bl = 0.f;                      // f0_n t_ap u
+    if (kAdjoint) {
+      const double p = r.f0[n] * r.t_ap * u;
+      bh = (float)p;
+      bl = (float)(p - (double)bh);
+    }
+    // samples [lo, hi) of a steady point have their four taps in the cube
+    const int lo = max(0, 1 - k0), hi = min(l, r.T - 2 - k0);
+    if (steady && (lo > 0 || hi < l)) edge |= l > 0;
+    const ChanPhase ph = s_ph[n];
+    const BlPhase bp = s_bl;
+    // offset + j step + rate (k0 + fr), modulo one cycle; the rate is signed
+    unsigned long long cyc = ph.offset + (unsigned long long)j * bp.step + (unsigned long long)(long long)k0 * ph.rate +
+                             (unsigned long long)ph.whole * fr64 + __umul64hi(ph.rate, fr64) -
+                             ((long long)ph.rate < 0 ? fr64 : 0ull);
+    const float2 *const src = vb + c;
+    float2 du = make_float2(0.f, 0.f);
+    // sample i with taps a0 .. a3 and phase ph_i
+    auto sample = [&](int i, unsigned long long ph_i, float2 a0, float2 a1, float2 a2, float2 a3) {
+      float red, fx = 0.f;
+      bool sure = round_fraction(ph_i, bp.slack8, bp.zmax, red);
+      if (kAdjoint) {
+        // f0_n t_ap (u + i) = (bh + bl) + i (f0h + f0l), to about 2^-44 of itself
+        float se;
+        const float fi = (float)i, p = __fmul_rn(fi, f0h), pe = fmaf(fi, f0h, -p);
+        const float sh = two_sum(bh, p, se), sl = se + (bl + fmaf(fi, f0l, pe)), d = fabsf(sh) * 0x1p-42f;
+        fx = sh + (sl - d);
+        sure = sure && fx == sh + (sl + d);
+      }
+      if (!sure) {
+        // the FP64 expressions, their operations spelled out (one branch for both: the shorter alone
+        // would be predicated, and predicated-off FP64 instructions take the pipe all the same)
+        const double x = opaque(u) + i;
+        const double f0n = r.f0[n];
+        const double fjd = __dmul_rn(__dmul_rn((double)j, r.f_bw), inv_j), fmd = __dsub_rn(f0n, r.f0_min);
+        const double rate = __dmul_rn(__dmul_rn(__dmul_rn(f0n, rho), r.t_ap), 1e-6);
+        const double cycles = __fma_rn(rate, x, __dmul_rn(__fma_rn(fjd, tau_s, __dmul_rn(fmd, tau_m)), 1e-3));
+        red = (float)__dsub_rn(cycles, floor(cycles));
+        if (kAdjoint) fx = (float)__dmul_rn(__dmul_rn(f0n, r.t_ap), x);
+      }
+      const float2 e = phasor(red);
+      const float2 smp = make_float2(fmaf(w[3], a3.x, fmaf(w[2], a2.x, fmaf(w[1], a1.x, w[0] * a0.x))),
+                                     fmaf(w[3], a3.y, fmaf(w[2], a2.y, fmaf(w[1], a1.y, w[0] * a0.y))));
+      const float2 t = cmulf(cmulf(wr, smp), e);
+      if (!kAdjoint) {
+        ac[0] += t.x;
+        ac[1] += t.y;
+        return;
+      }
+      const float2 dsmp = make_float2(fmaf(dw[3], a3.x, fmaf(dw[2], a2.x, fmaf(dw[1], a1.x, dw[0] * a0.x))),
+                                      fmaf(dw[3], a3.y, fmaf(dw[2], a2.y, fmaf(dw[1], a1.y, dw[0] * a0.y))));
+      ac[0] = fmaf(t.x, pt.fj, ac[0]);
+      ac[1] = fmaf(t.y, pt.fj, ac[1]);
+      ac[2] = fmaf(t.x, pt.fm, ac[2]);
+      ac[3] = fmaf(t.y, pt.fm, ac[3]);
+      ac[4] = fmaf(t.x, fx, ac[4]);
+      ac[5] = fmaf(t.y, fx, ac[5]);
+      // d/du of the sample: c X'(x) e^{-i Phi} + t (-i dPhi/du), dPhi/du = 2 pi f0_n rho t_ap 1e-6
+      const float2 td = cmulf(cmulf(wr, dsmp), e);
+      du.x += fmaf(ph.arate, t.y, td.x);
+      du.y += fmaf(-ph.arate, t.x, td.y);
+    };
+    if (steady) {
+      // the taps slide; those of kRefAhead samples are loaded ahead of their arithmetic
+      if (lo < hi) {
+        cyc += (unsigned long long)lo * ph.rate;
+        const float2 *s = src + (size_t)(k0 - 1 + lo) * r.C;
+        float2 v[3 + kRefAhead];
+#pragma unroll
+        for (int q = 0; q < 3; ++q, s += r.C) v[q] = __ldg(s);
+        for (int i = lo; i < hi; i += kRefAhead) {
+#pragma unroll
+          for (int q = 0; q < kRefAhead; ++q, s += r.C) v[3 + q] = i + q < hi ? __ldg(s) : make_float2(0.f, 0.f);
+#pragma unroll
+          for (int q = 0; q < kRefAhead; ++q, cyc += ph.rate)
+            if (i + q < hi) sample(i + q, cyc, v[q], v[q + 1], v[q + 2], v[q + 3]);
+#pragma unroll
+          for (int q = 0; q < 3; ++q) v[q] = v[kRefAhead + q];
+        }
+      }
+    } else {
+      for (int i = 0; i < l; ++i, cyc += ph.rate) {
+        const double x = u + i;
+        const int k = __double2int_rd(x);  // saturates
+        if (k < 1 || k > r.T - 3) {
+          edge = true;
+          continue;
+        }
+        cr_weights((float)(x - floor(x)), w, dw);
+        const float2 *s = src + (size_t)(k - 1) * r.C;
+        sample(i, cyc, __ldg(s), __ldg(s + r.C), __ldg(s + 2 * (size_t)r.C), __ldg(s + 3 * (size_t)r.C));
+      }
+    }
+    if (kAdjoint) {
+      ac[6] += du.x;
+      ac[7] += du.y;
+      ac[8] = fmaf(du.x, pt.df, ac[8]);
+      ac[9] = fmaf(du.y, pt.df, ac[9]);
+    }
+  }
+  block_sum<kVals>(ac, red, sums);
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(kRefThreads) k_refine_fwd(RefineArgs r) {
-  __shared__ float red[2 * 32];
+__global__ void __launch_bounds__(kRefThreads, 4) k_refine_fwd(const __grid_constant__ RefineArgs r) {
+  __shared__ float sums[2];
   const int cand = blockIdx.x, b = blockIdx.y;
-  const double *th = r.params + (size_t)cand * r.n_par;
-  const double dm = th[0], t0 = th[1], tau_s = th[2 + 3 * b], tau_m = th[3 + 3 * b], rho = th[4 + 3 * b];
-  const int l = r.width[cand];
-  const float2 *vb = r.vis + (size_t)b * r.T * r.C;
-  float acc[2] = {0.f, 0.f};
   bool edge = false;
-  for (int c = threadIdx.x; c < r.C; c += blockDim.x) {
-    const PointConst p = point_const(r, c);
-    if (p.wrot.x == 0.f && p.wrot.y == 0.f) continue;  // j = 0 or flagged
-    const double u = t0 + dm * p.ddm;
-    const double base = (p.fj * tau_s + p.fmbd * tau_m) * 1e-3;
-    const double rate = p.f0n * rho * r.t_ap * 1e-6;
-    for (int i = 0; i < l; ++i) {
-      const double x = u + i;
-      const double kf = floor(x);
-      const long long k = (long long)kf;
-      if (k - 1 < 0 || k + 2 > r.T - 1) {
-        edge = true;
-        continue;
-      }
-      float w[4], dw[4];
-      cr_weights((float)(x - kf), w, dw);
-      const float2 *s = vb + (size_t)(k - 1) * r.C + c;
-      float2 smp = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const float2 v = __ldg(s + (size_t)m * r.C);
-        smp.x = fmaf(w[m], v.x, smp.x);
-        smp.y = fmaf(w[m], v.y, smp.y);
-      }
-      const float2 t = cmulf(cmulf(p.wrot, smp), phasor(base + rate * x));
-      acc[0] += t.x;
-      acc[1] += t.y;
-    }
-  }
+  refine_walk<false>(r, cand, b, sums, edge);
   if (edge) r.status[cand] = 1;
-  block_sum<2>(acc, red);
-  if (threadIdx.x == 0) {
-    r.g[2 * ((size_t)cand * r.n_bl + b)] = acc[0];
-    r.g[2 * ((size_t)cand * r.n_bl + b) + 1] = acc[1];
-  }
+  if (threadIdx.x < 2) r.g[2 * ((size_t)cand * r.n_bl + b) + threadIdx.x] = sums[threadIdx.x];
 }
 
 __global__ void k_refine_power(RefineArgs r) {
@@ -138,62 +322,11 @@ __global__ void k_refine_power(RefineArgs r) {
   r.power[cand] = p;
 }
 
-__global__ void __launch_bounds__(kRefThreads) k_refine_adjoint(RefineArgs r) {
-  __shared__ float red[10 * 32];
+__global__ void __launch_bounds__(kRefThreads, 3) k_refine_adjoint(const __grid_constant__ RefineArgs r) {
+  __shared__ float acc[10];
   const int cand = blockIdx.x, b = blockIdx.y;
-  const double *th = r.params + (size_t)cand * r.n_par;
-  const double dm = th[0], t0 = th[1], tau_s = th[2 + 3 * b], tau_m = th[3 + 3 * b], rho = th[4 + 3 * b];
-  const int l = r.width[cand];
-  const float2 *vb = r.vis + (size_t)b * r.T * r.C;
-  // sums: term * f_j, term * fmbd, term * f0n t_ap x, dG/du, dG/du * ddm (complex each)
-  float acc[10];
-#pragma unroll
-  for (int k = 0; k < 10; ++k) acc[k] = 0.f;
-  for (int c = threadIdx.x; c < r.C; c += blockDim.x) {
-    const PointConst p = point_const(r, c);
-    if (p.wrot.x == 0.f && p.wrot.y == 0.f) continue;
-    const double u = t0 + dm * p.ddm;
-    const double base = (p.fj * tau_s + p.fmbd * tau_m) * 1e-3;
-    const double rate = p.f0n * rho * r.t_ap * 1e-6;
-    const float arate = (float)(6.283185307179586 * p.f0n * rho * r.t_ap * 1e-6);  // dPhi/du
-    float2 du_sum = make_float2(0.f, 0.f);
-    for (int i = 0; i < l; ++i) {
-      const double x = u + i;
-      const double kf = floor(x);
-      const long long k = (long long)kf;
-      if (k - 1 < 0 || k + 2 > r.T - 1) continue;
-      float w[4], dw[4];
-      cr_weights((float)(x - kf), w, dw);
-      const float2 *s = vb + (size_t)(k - 1) * r.C + c;
-      float2 smp = make_float2(0.f, 0.f), dsmp = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const float2 v = __ldg(s + (size_t)m * r.C);
-        smp.x = fmaf(w[m], v.x, smp.x);
-        smp.y = fmaf(w[m], v.y, smp.y);
-        dsmp.x = fmaf(dw[m], v.x, dsmp.x);
-        dsmp.y = fmaf(dw[m], v.y, dsmp.y);
-      }
-      const float2 e = phasor(base + rate * x);
-      const float2 t = cmulf(cmulf(p.wrot, smp), e);
-      const float fj = (float)p.fj, fm = (float)p.fmbd, fx = (float)(p.f0n * r.t_ap * x);
-      acc[0] = fmaf(t.x, fj, acc[0]);
-      acc[1] = fmaf(t.y, fj, acc[1]);
-      acc[2] = fmaf(t.x, fm, acc[2]);
-      acc[3] = fmaf(t.y, fm, acc[3]);
-      acc[4] = fmaf(t.x, fx, acc[4]);
-      acc[5] = fmaf(t.y, fx, acc[5]);
-      // d/du of the sample: c X'(x) e^{-i Phi} + t (-i dPhi/du), dPhi/du = 2 pi f0_n rho t_ap 1e-6
-      const float2 td = cmulf(cmulf(p.wrot, dsmp), e);
-      du_sum.x += td.x + arate * t.y;
-      du_sum.y += td.y - arate * t.x;
-    }
-    acc[6] += du_sum.x;
-    acc[7] += du_sum.y;
-    acc[8] = fmaf(du_sum.x, (float)p.ddm, acc[8]);
-    acc[9] = fmaf(du_sum.y, (float)p.ddm, acc[9]);
-  }
-  block_sum<10>(acc, red);
+  bool edge = false;
+  refine_walk<true>(r, cand, b, acc, edge);
   if (threadIdx.x == 0) {
     const float gr = r.g[2 * ((size_t)cand * r.n_bl + b)], gi = r.g[2 * ((size_t)cand * r.n_bl + b) + 1];
     const float up = r.dpower[cand];
