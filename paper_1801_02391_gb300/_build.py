@@ -14,7 +14,7 @@ LIB = os.path.join(OUT_DIR, "libfrbx.so")
 # peak-rate probes of the GPU (roofline denominators of the bench), a library of their own
 LIB_PEAKS = os.path.join(OUT_DIR, "libfrbx_peaks.so")
 PEAKS_SOURCES = ["peaks.cu"]
-SOURCES = ["frbx_api.cu", "kernels_fit.cu", "kernels_fft.cu", "kernels_mma.cu", "kernels_misc.cu", "kernels_refine.cu", "kernels_calib.cu", "kernels_tree.cu", "kernels_tree_mma.cu", "noalloc.cu", "extract.cpp"]
+SOURCES = ["frbx_api.cu", "kernels_fit.cu", "kernels_fft.cu", "kernels_mma.cu", "kernels_misc.cu", "kernels_refine.cu", "kernels_calib.cu", "kernels_tree.cu", "kernels_tree16.cu", "kernels_tree_mma.cu", "noalloc.cu", "extract.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-ffp-contract=off",
               "-I", os.path.join(ROOT, "include")]

@@ -31,6 +31,20 @@ __host__ __device__ constexpr int bitrev5(int k) {
   return ((k & 1) << 4) | ((k & 2) << 2) | (k & 4) | ((k & 8) >> 2) | ((k & 16) >> 4);
 }
 
+// Packed per-thread key of a cell, |G|^2 with its low mantissa bits replaced by a code that
+// prefers the lower q2 on equal truncated powers.  Whole grid: 4 bits, 15 - b with b = q2 div 2
+// the thread's cell rank (2^-19 relative truncation; between the two threads of a class the
+// even half h = 0 wins a tie as the lower lane), merged by one lop3 with m = ~15 kept in a
+// register.  Delay windows (fewer registers to spare): 6 bits, 32 - q2 (2^-17).
+template <bool kFull>
+__device__ __forceinline__ unsigned cell_key(float2 v, int b, int h, unsigned m) {
+  const float p = fmaf(v.x, v.x, v.y * v.y);
+  if constexpr (!kFull) return (__float_as_uint(p) & ~63u) | (unsigned)(32 - (2 * b + h));
+  unsigned d;
+  asm("lop3.b32 %0, %1, %2, %3, 0xE4;" : "=r"(d) : "r"(__float_as_uint(p)), "r"(15u - (unsigned)b), "r"(m));
+  return d;
+}
+
 struct Seg {
   int bl, d, l, k0;
   long long out;

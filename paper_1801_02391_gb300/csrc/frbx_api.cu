@@ -829,12 +829,20 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
   for (int b = 0; b < n_bl; ++b)
     for (int d = 0; d < n_dm; ++d)
       if (T - dkm[(size_t)d] >= 1) r->ser.push_back(make_int2(b, d));
+  if (!mma && frbx::tree16_supported(h->Ls, h->Lm, h->N, h->J, h->tree_s16, h->g.data(), T)) {
+    // both passes in one kernel: no spectra in device memory, a time tile of its own
+    t.fused = 1;
+    t.TT = frbx::tree16_tile(h->Ls, T, (long long)r->ser.size());
+    t.n_tt = (T + t.TT - 1) / t.TT;
+    t.y_series = 0;
+  }
   // per series: its transformed spectra, the E4M3 form's per-AP scales and the deep anchors of
   // its MBD CTAs
-  const size_t anc_per = mma ? 0 : sizeof(float2) * frbx::tree_anchor_floats(nlev) * t.n_mb * t.n_tt;
+  const size_t anc_per = mma || t.fused ? 0 : sizeof(float2) * frbx::tree_anchor_floats(nlev) * t.n_mb * t.n_tt;
   const size_t sc_per = form == 2 ? sizeof(float) * (size_t)T : 0;
   const size_t per = sizeof(float2) * t.y_series + sc_per + anc_per;
-  r->chunk = std::max<size_t>(1, std::min(std::max<size_t>(r->ser.size(), 1), budget / per));
+  const size_t all = std::max<size_t>(r->ser.size(), 1);
+  r->chunk = t.fused ? all : std::max<size_t>(1, std::min(all, budget / per));
   r->sc_off = (sizeof(float2) * t.y_series * r->chunk + 255) & ~(size_t)255;
   r->y_bytes = r->sc_off + ((sc_per * r->chunk + 255) & ~(size_t)255);
   r->a_bytes = (anc_per * r->chunk + 255) & ~(size_t)255;
@@ -885,14 +893,15 @@ int enqueue_tree(frbx_handle *h, const FitArgs &a, const TreeRun &r, const int2 
       if (ci >= 2) e = cudaStreamWaitEvent(sA, evB[par], 0);  // the MBD pass two chunks back is done with this set
       if (e == cudaSuccess && copied) e = cudaStreamWaitEvent(sA, copied[r.ser[c0 + (size_t)tc.n_s - 1].x], 0);
       if (e == cudaSuccess && kev) e = cudaEventRecord(kev[0], sA);
-      if (e == cudaSuccess) e = frbx::launch_tree_sbd(a, tc, sA, &h->launches);
+      if (e == cudaSuccess && !t.fused) e = frbx::launch_tree_sbd(a, tc, sA, &h->launches);
       if (e == cudaSuccess && kev) e = cudaEventRecord(kev[1], sA);
       if (e == cudaSuccess) e = cudaEventRecord(evA[par], sA);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(sB, evA[par], 0);
       if (e == cudaSuccess && kev) e = cudaEventRecord(kev[2], sB);
       if (e == cudaSuccess)
-        e = t.mma ? frbx::launch_tree_mma(tc, r.full, sB, &h->launches)
-                  : frbx::launch_tree_mbd(tc, r.full, sB, &h->launches);
+        e = t.mma     ? frbx::launch_tree_mma(tc, r.full, sB, &h->launches)
+            : t.fused ? frbx::launch_tree16(a, tc, r.full, sB, &h->launches)
+                      : frbx::launch_tree_mbd(tc, r.full, sB, &h->launches);
       if (e == cudaSuccess && kev) e = cudaEventRecord(kev[3], sB);
       if (e == cudaSuccess) e = cudaEventRecord(evB[par], sB);
       if (e == cudaErrorInvalidConfiguration) return fail(h, FRBX_EUNSUPPORTED, "window-tree fit does not fit this shape");
@@ -1824,7 +1833,7 @@ extern "C" int frbx_search_batch(frbx_batch *b, const frbx_scan *scans, int32_t 
         TreeRun r;
         plan_tree(h, a, tree_lev[g], windows, n_win, dkm[g], scans[i_g].n_bl, scans[i_g].T, n_dm, a.win_off, a.S_tot,
                   tree_budget(h), tree_tc[g] != 0 ? 0 : -1, &r, TT);
-        if (r.ser.empty()) break;
+        if (r.ser.empty() || r.t.fused) break;  // the fused kernel takes a tile of its own
         r.ser.resize(std::min(r.ser.size(), r.chunk));
         if (ensure(h, h->ytree, r.need()) != cudaSuccess || tree_prepare(h) != FRBX_OK) {
           cudaGetLastError();
@@ -1865,7 +1874,7 @@ extern "C" int frbx_search_batch(frbx_batch *b, const frbx_scan *scans, int32_t 
       need_h[(size_t)g] = std::max(need_h[(size_t)g], truns[(size_t)i].need());
       tser_off[(size_t)i] = tser_all.size();
       tser_all.insert(tser_all.end(), truns[(size_t)i].ser.begin(), truns[(size_t)i].ser.end());
-      tree_launches += 2 * (int64_t)((truns[(size_t)i].ser.size() + truns[(size_t)i].chunk - 1) / truns[(size_t)i].chunk) + 1;
+      tree_launches += (truns[(size_t)i].t.fused ? 1 : 2) * (int64_t)((truns[(size_t)i].ser.size() + truns[(size_t)i].chunk - 1) / truns[(size_t)i].chunk) + 1;
     }
     for (size_t g = 0; g < setups.size(); ++g) {
       if (tree_lev[g] < 0) continue;

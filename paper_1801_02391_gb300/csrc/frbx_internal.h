@@ -168,6 +168,7 @@ struct TreeArgs {
   int n_dm, S_tot;
   const int *win_off;      // [n_win]
   int N, NS, Ls, Lm, PM, RB, n_mb, TT, n_tt, nlev;
+  int fused;               // k_tree16 runs both passes (no Y)
   int half;                // k_tree_mbd with Lm = 16: one thread per SBD row, its 16 cells q = 0..15
   int emit_w[8];           // window index of level e (window 2^e), -1 = not searched
   int m_lo, m_len, q_lo, q_len;
@@ -215,6 +216,12 @@ cudaError_t launch_tree_finalize(frbx_seg *series, long long n_el, int S_tot, in
                                  const int *win_off, const int *n_valid, int log2Lm, int Lm, cudaStream_t st,
                                  int64_t *launches);
 void set_tree_constants();
+
+// kernels_tree16.cu: both passes of the FP32 window tree in one kernel, 16-column grids
+bool tree16_supported(int Ls, int Lm, int N, int J, int s16, const int *g, int T);
+int tree16_tile(int Ls, int T, long long n_series);  // its time tile
+cudaError_t launch_tree16(const FitArgs &a, const TreeArgs &t, bool full, cudaStream_t st, int64_t *launches);
+void set_tree16_constants();
 
 // kernels_misc.cu
 cudaError_t launch_shift_table(const double *f, int C, double fref, const double *dm, int n_dm,

@@ -152,6 +152,7 @@ void set_fft_constants() {
   upload_w32();
   set_mma_constants();
   set_tree_constants();
+  set_tree16_constants();
 }
 
 bool fft_supported(int Ls, int Lm, int J) { return Ls % 32 == 0 && Lm % 32 == 0 && J <= Ls; }

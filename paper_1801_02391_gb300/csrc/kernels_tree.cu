@@ -254,20 +254,6 @@ __global__ void __launch_bounds__(kTreeThreads, 4)
 }
 
 // ----------------------------------------------------------------------------- MBD + tree
-// Packed per-thread key of a cell, |G|^2 with its low mantissa bits replaced by a code that
-// prefers the lower q2 on equal truncated powers.  Whole grid: 4 bits, 15 - b with b = q2 div 2
-// the thread's cell rank (2^-19 relative truncation; between the two threads of a class the
-// even half h = 0 wins a tie as the lower lane), merged by one lop3 with m = ~15 kept in a
-// register.  Delay windows (fewer registers to spare): 6 bits, 32 - q2 (2^-17).
-template <bool kFull>
-__device__ __forceinline__ unsigned cell_key(float2 v, int b, int h, unsigned m) {
-  const float p = fmaf(v.x, v.x, v.y * v.y);
-  if constexpr (!kFull) return (__float_as_uint(p) & ~63u) | (unsigned)(32 - (2 * b + h));
-  unsigned d;
-  asm("lop3.b32 %0, %1, %2, %3, 0xE4;" : "=r"(d) : "r"(__float_as_uint(p)), "r"(15u - (unsigned)b), "r"(m));
-  return d;
-}
-
 template <int S16, bool kFull>
 __global__ void __launch_bounds__(kTreeThreads, 3) k_tree_mbd(const __grid_constant__ TreeArgs t) {
   extern __shared__ __align__(16) unsigned char smem[];
