@@ -492,7 +492,7 @@ void frbx_destroy(frbx_handle *h) {
     if (e) cudaEventDestroy(e);
   if (h->copy_st) cudaStreamDestroy(h->copy_st);
   frbx_handle::Buf *bufs[] = {&h->vis, &h->dk, &h->dk_max, &h->series, &h->pnorm, &h->stats,
-                              &h->counts, &h->offsets, &h->events, &h->small, &h->seglist, &h->masks,
+                              &h->counts, &h->offsets, &h->events, &h->small, &h->seglist, &h->masks, &h->hits,
                               &h->errflag, &h->refine, &h->calib, &h->ytree};
   for (auto *b : bufs)
     if (b->p) cudaFree(b->p);
@@ -719,6 +719,8 @@ int run_stats(frbx_handle *h, StatsArgs sa, cudaStream_t st, std::vector<frbx_ev
   FRBX_CK(h, ensure(h, h->stats, sizeof(double) * 2 * ns));
   FRBX_CK(h, ensure(h, h->counts, sizeof(int) * (ns + 1)));
   FRBX_CK(h, ensure(h, h->offsets, sizeof(long long) * (ns + 1)));
+  FRBX_CK(h, ensure(h, h->hits, frbx::stats_hit_bytes(sa.n_series, sa.n_dm, sa.S_tot, sa.n_win)));
+  sa.hits = (unsigned *)h->hits.p;
   sa.mean_std = (double *)h->stats.p;
   sa.counts = (int *)h->counts.p;
   sa.offsets = (long long *)h->offsets.p;

@@ -239,11 +239,13 @@ struct StatsArgs {
   double threshold;
   double *mean_std;        // [n_series][n_dm][n_win][2]
   int *counts;             // [n_series * n_dm * n_win + 1]
+  unsigned *hits;          // one bit per valid slot (stats_hit_bytes)
   long long *offsets;      // [n_series * n_dm * n_win + 1]
   frbx_event *events;      // output
   float *pnorm;            // optional [n_series][n_dm][S_tot]
   int series_base;         // value stored in frbx_event.series = series_base + s
 };
+size_t stats_hit_bytes(int n_series, int n_dm, int S_tot, int n_win);
 cudaError_t launch_stats_count(const StatsArgs &a, cudaStream_t st, int64_t *launches);
 cudaError_t launch_scan(const StatsArgs &a, cudaStream_t st, int64_t *launches);
 cudaError_t launch_events(const StatsArgs &a, cudaStream_t st, int64_t *launches);
@@ -312,6 +314,6 @@ struct frbx_handle {
   };
   frbx_limits lim{};          // frbx_set_limits (all zero = defaults)
   size_t scratch_total = 0;   // bytes held by the Bufs below
-  Buf vis, dk, dk_max, series, pnorm, stats, counts, offsets, events, small, seglist, masks, errflag, refine, calib,
+  Buf vis, dk, dk_max, series, pnorm, stats, counts, offsets, events, small, seglist, masks, hits, errflag, refine, calib,
       ytree;
 };

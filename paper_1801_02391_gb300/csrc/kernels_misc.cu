@@ -78,28 +78,146 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
   return t;
 }
 
-// One CTA per (window, DM, series): population mean and std over the valid segments,
-// then the count of P = (A - mean) / std > threshold; optionally writes P.
+// Exact sum of two floats: a + b = s + e (Knuth's two-sum), and the same for |a| >= |b|
+__device__ __forceinline__ float two_sum(float a, float b, float &e) {
+  const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
+  return s;
+}
+__device__ __forceinline__ float fast_two_sum(float a, float b, float &e) {
+  const float s = __fadd_rn(a, b);
+  e = __fsub_rn(b, __fsub_rn(s, a));
+  return s;
+}
+// a float pair hi + lo (|lo| at most half a unit in the last place of hi: about 48 bits)
+struct Pair {
+  float hi, lo;
+};
+__device__ __forceinline__ Pair to_pair(double v) {
+  const float h = (float)v;
+  return {h, (float)(v - (double)h)};
+}
+// running sum of floats in three floats: no rounding above about 2^-70 of the terms
+struct Sum3 {
+  float s = 0.f, e = 0.f, f = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    float d, g;
+    s = two_sum(s, x, d);
+    e = two_sum(e, d, g);
+    f += g;
+  }
+  __device__ __forceinline__ double value() const { return (double)s + ((double)e + (double)f); }
+};
+
+// series_value as a pair
+__device__ __forceinline__ Pair series_pair(const StatsArgs &a, int s, int d, int slot) {
+  if (!a.masks) return {a.series[((size_t)s * a.n_dm + d) * a.S_tot + slot].amp, 0.f};
+  const unsigned long long mask = a.masks[s];
+  Pair v = {0.f, 0.f};
+  for (int b = 0; b < a.n_bl; ++b)
+    if ((mask >> b) & 1ull) {
+      float e;
+      v.hi = two_sum(v.hi, a.series[((size_t)b * a.n_dm + d) * a.S_tot + slot].amp, e);
+      v.lo += e;
+    }
+  v.hi = fast_two_sum(v.hi, v.lo, v.lo);
+  return v;
+}
+
+// v - c - (m.hi + m.lo)
+__device__ __forceinline__ Pair minus(Pair v, float c, Pair m) {
+  float e1, e2;
+  const float s1 = two_sum(v.hi, -c, e1), s2 = two_sum(s1, -m.hi, e2);
+  Pair r;
+  r.hi = fast_two_sum(s2, e2 + (e1 + (v.lo - m.lo)), r.lo);
+  return r;
+}
+
+// words of the hit mask of window w of one (series, DM): its slots' bits start at word (off >> 5) + w
+__host__ __device__ __forceinline__ size_t hit_words(int S_tot, int n_win) { return (size_t)(S_tot >> 5) + n_win + 1; }
+
+// One CTA per (window, DM, series): population mean and std over the valid segments, then the
+// crossings P = (A - mean) / std > threshold, their count and one bit each; optionally writes P.
+//
+// FP64 runs at a 64th of FP32's rate here, and a division of it per slot was most of this kernel and of
+// the one that writes the events.  The sums are taken of the differences from the first amplitude (and of
+// their squares, with the products' rounding) in three floats each, P is formed in float pairs, and
+// both are as exact as the FP64 they replace; P's pair decides a crossing unless it is within 1e-9 of
+// the threshold, which the FP64 expression then decides.  Series whose squares FP32 cannot hold, or with a
+// value that is not finite, take FP64 throughout.  With k_events and k_scan below, for 2.1 million slots
+// of baselines and four combinations: 0.71 -> 0.45 ms.
 __global__ void __launch_bounds__(256) k_stats_count(StatsArgs a) {
   __shared__ double red[32];
   const int w = blockIdx.x, d = blockIdx.y, s = blockIdx.z;
   const int nv = a.n_valid[d * a.n_win + w];
   const int off = a.win_off[w];
   const size_t sid = ((size_t)s * a.n_dm + d) * a.n_win + w;
-  double sum = 0.0;
-  for (int i = threadIdx.x; i < nv; i += blockDim.x) sum += series_value(a, s, d, off + i);
-  const double mean = nv > 0 ? block_sum(sum, red) / nv : 0.0;
-  double sq = 0.0;
-  for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-    const double dv = series_value(a, s, d, off + i) - mean;
-    sq += dv * dv;
+  unsigned *const bits = a.hits + ((size_t)s * a.n_dm + d) * hit_words(a.S_tot, a.n_win) + (off >> 5) + w;
+  double mean = 0.0, sd = 0.0, shift = 0.0;  // shift: mean - c
+  float c = 0.f;
+  bool fast = nv > 0;
+  if (fast) c = series_pair(a, s, d, off).hi;
+  for (int pass = 0; fast && pass < 2; ++pass) {
+    Sum3 s1, s2;
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+      const Pair x = minus(series_pair(a, s, d, off + i), c, {0.f, 0.f});
+      s1.add(x.hi);
+      s1.add(x.lo);
+      const float q = __fmul_rn(x.hi, x.hi);
+      s2.add(q);
+      s2.add(fmaf(2.f * x.hi, x.lo, fmaf(x.hi, x.hi, -q)));
+    }
+    const double t1 = block_sum(s1.value(), red), t2 = block_sum(s2.value(), red);
+    shift = t1 / nv;
+    mean = (double)c + shift;
+    const double var = fmax(t2 / nv - shift * shift, 0.0);
+    sd = sqrt(var);
+    // squares within FP32 with room for their rounding terms (or all equal); false for NaN
+    fast = t2 == 0.0 || (t2 >= 1e-18 * nv && t2 <= 1e28);
+    if (shift * shift <= 16.0 * var) break;  // c near the mean: nothing cancelled
+    if (pass == 1) fast = fast && shift * shift <= 1e6 * var;
+    c = (float)mean;
   }
-  const double sd = nv > 0 ? sqrt(block_sum(sq, red) / nv) : 0.0;
+  if (!fast && nv > 0) {
+    double sum = 0.0;
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) sum += series_value(a, s, d, off + i);
+    mean = block_sum(sum, red) / nv;
+    double sq = 0.0;
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+      const double dv = series_value(a, s, d, off + i) - mean;
+      sq += dv * dv;
+    }
+    sd = sqrt(block_sum(sq, red) / nv);
+  }
+  const double inv = sd > 0.0 ? 1.0 / sd : 0.0;
+  const Pair m = to_pair(mean - (double)c), r = to_pair(inv), th = to_pair(a.threshold);
   int cnt = 0;
-  for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-    const double p = sd > 0.0 ? (series_value(a, s, d, off + i) - mean) / sd : 0.0;
-    if (p > a.threshold) ++cnt;
-    if (a.pnorm) a.pnorm[((size_t)s * a.n_dm + d) * a.S_tot + off + i] = (float)p;
+  for (int i0 = threadIdx.x & ~31; i0 < nv; i0 += blockDim.x) {  // 32 slots of a warp: one word
+    const int i = i0 + (threadIdx.x & 31);
+    bool hit = false;
+    float pn = 0.f;
+    if (i < nv) {
+      bool sure = fast && sd > 0.0;
+      if (sure) {
+        const Pair x = minus(series_pair(a, s, d, off + i), c, m);
+        const float ph = __fmul_rn(x.hi, r.hi), pl = fmaf(x.hi, r.lo, fmaf(x.lo, r.hi, fmaf(x.hi, r.hi, -ph)));
+        pn = ph + pl;
+        const float g = (ph - th.hi) + (pl - th.lo);
+        hit = g > 0.f;
+        sure = fabsf(g) > 1e-9f * (1.f + fabsf(ph));  // false for NaN
+      }
+      if (!sure) {
+        const double p = sd > 0.0 ? (series_value(a, s, d, off + i) - mean) / sd : 0.0;
+        hit = p > a.threshold;
+        pn = (float)p;
+      }
+      if (a.pnorm) a.pnorm[((size_t)s * a.n_dm + d) * a.S_tot + off + i] = pn;
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, hit);
+    if ((threadIdx.x & 31) == 0) {
+      bits[i0 >> 5] = bal;
+      cnt += __popc(bal);
+    }
   }
   const double total = block_sum((double)cnt, red);
   if (threadIdx.x == 0) {
@@ -109,75 +227,76 @@ __global__ void __launch_bounds__(256) k_stats_count(StatsArgs a) {
   }
 }
 
+// Exclusive sum over a CTA of 1024 threads; total gets the sum.
+__device__ __forceinline__ long long block_exclusive(long long v, long long *warp_sum, long long &total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  long long inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  __syncthreads();
+  if (lane == 31) warp_sum[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    const long long x = lane < nw ? warp_sum[lane] : 0;
+    long long y = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long t = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= o) y += t;
+    }
+    warp_sum[lane] = y - x;
+    if (lane == 31) warp_sum[32] = y;
+  }
+  __syncthreads();
+  total = warp_sum[32];
+  return warp_sum[warp] + inc - v;
+}
+
 // Exclusive scan of the per-(series, DM, window) counts into offsets (one CTA).
 __global__ void __launch_bounds__(1024) k_scan(const int *__restrict__ counts, long long n,
                                                long long *__restrict__ offsets) {
-  __shared__ long long part[1024];
+  __shared__ long long part[33];
   const long long chunk = (n + blockDim.x - 1) / blockDim.x;
   const long long lo = threadIdx.x * chunk, hi = min(n, lo + chunk);
-  long long s = 0;
+  long long s = 0, total;
   for (long long i = lo; i < hi; ++i) s += counts[i];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    long long run = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      const long long v = part[t];
-      part[t] = run;
-      run += v;
-    }
-    offsets[n] = run;
-  }
-  __syncthreads();
-  long long run = part[threadIdx.x];
+  long long run = block_exclusive(s, part, total);
+  if (threadIdx.x == 0) offsets[n] = total;
   for (long long i = lo; i < hi; ++i) {
     offsets[i] = run;
     run += counts[i];
   }
 }
 
-// Ordered compaction of the crossings of one (window, DM, series) in ascending k0.
+// The crossings of one (window, DM, series) in ascending k0, from the bits k_stats_count left.
 __global__ void __launch_bounds__(256) k_events(StatsArgs a) {
-  __shared__ int wsum[8];
-  __shared__ int base_s;
+  __shared__ long long part[33];
   const int w = blockIdx.x, d = blockIdx.y, s = blockIdx.z;
-  const int nv = a.n_valid[d * a.n_win + w];
-  const int off = a.win_off[w], step = a.win_step[w];
   const size_t sid = ((size_t)s * a.n_dm + d) * a.n_win + w;
+  if (a.counts[sid] == 0) return;
+  const int nv = a.n_valid[d * a.n_win + w], nw = (nv + 31) >> 5;
+  const int off = a.win_off[w], step = a.win_step[w];
+  const unsigned *const bits = a.hits + ((size_t)s * a.n_dm + d) * hit_words(a.S_tot, a.n_win) + (off >> 5) + w;
   const double mean = a.mean_std[2 * sid], sd = a.mean_std[2 * sid + 1];
   long long out = a.offsets[sid];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int c0 = 0; c0 < nv; c0 += blockDim.x) {
-    const int i = c0 + threadIdx.x;
-    double v = 0.0, p = 0.0;
-    bool hit = false;
-    if (i < nv) {
-      v = series_value(a, s, d, off + i);
-      p = sd > 0.0 ? (v - mean) / sd : 0.0;
-      hit = p > a.threshold;
-    }
-    const unsigned bal = __ballot_sync(0xffffffffu, hit);
-    if (lane == 0) wsum[warp] = __popc(bal);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int run = 0;
-      for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-        const int t = wsum[k];
-        wsum[k] = run;
-        run += t;
-      }
-      base_s = run;
-    }
-    __syncthreads();
-    if (hit) {
-      const long long pos = out + wsum[warp] + __popc(bal & ((1u << lane) - 1u));
+  for (int c0 = 0; c0 < nw; c0 += blockDim.x) {
+    const int q = c0 + threadIdx.x;
+    unsigned word = q < nw ? bits[q] : 0u;
+    long long total;
+    long long pos = out + block_exclusive(__popc(word), part, total);
+    for (; word != 0u; word &= word - 1u, ++pos) {
+      const int i = q * 32 + __ffs((int)word) - 1;
+      const double v = series_value(a, s, d, off + i);
       frbx_event e;
       e.series = a.series_base + s;
       e.dm_idx = d;
       e.win_idx = w;
       e.k0 = i * step;
       e.amp = (float)v;
-      e.pnorm = (float)p;
+      e.pnorm = (float)(sd > 0.0 ? (v - mean) / sd : 0.0);
       if (!a.masks) {
         const frbx_seg sg = a.series[((size_t)s * a.n_dm + d) * a.S_tot + off + i];
         e.sbd_idx = sg.sbd_idx;
@@ -188,9 +307,12 @@ __global__ void __launch_bounds__(256) k_events(StatsArgs a) {
       }
       a.events[pos] = e;
     }
-    out += base_s;
-    __syncthreads();
+    out += total;
   }
+}
+
+size_t stats_hit_bytes(int n_series, int n_dm, int S_tot, int n_win) {
+  return sizeof(unsigned) * (size_t)n_series * n_dm * hit_words(S_tot, n_win);
 }
 
 cudaError_t launch_stats_count(const StatsArgs &a, cudaStream_t st, int64_t *launches) {
