@@ -748,7 +748,8 @@ int run_stats(frbx_handle *h, StatsArgs sa, cudaStream_t st, std::vector<frbx_ev
 // keys, zeroed first); a last pass turns the keys into frbx_seg records.  d_tab holds the
 // window tables and valid-segment counts in the layout frbx_search uploads.
 // Time tile of the window-tree fit (APs per MBD CTA, a multiple of 64; frbx_search doubles it
-// for long scans on the tensor cores); frbx_search_batch measures the candidates per setup.
+// for long scans on the tensor cores and takes packed_time_tile's with packed delay windows);
+// frbx_search_batch measures the candidates per setup.
 constexpr int kTreeTT = 1024;
 constexpr int kTreeTuneTT[] = {512, 1024, 2048};
 
@@ -762,12 +763,36 @@ struct TreeRun {
   size_t need() const { return 2 * (y_bytes + a_bytes); }  // two buffer sets: chunks alternate
 };
 
+// Time tile of a tensor-core MBD launch of n_s series with packed delay windows: one CTA per SM walks pack
+// tiles side by side, so a launch takes rounds(CTAs / SMs) times the APs of a tile, the lmax - 1 trailing
+// APs it repeats and about kCtaAps APs' time of setup.  Tiles of equal length (t_max: APs of the longest
+// sweep-free stretch), a multiple of pack of them, in the number that makes this least.  Fixed tiles left
+// pieces empty: 9973 APs in 2048-AP tiles are five, so the second group of four held one.  32 x 3 series
+// with a +-64 ns window: 37.0 -> 32.2 ms.  (Whole tiles gain nothing from it: short last tiles
+// fill the ends of the rounds.)
+constexpr int kCtaAps = 12;
+int packed_time_tile(int t_max, int pack, int n_s, int n_qb, int lmax) {
+  const long long sms = frbx::sm_count();
+  long long best = INT64_MAX;
+  int tile = 64;
+  for (int ng = 1;; ++ng) {
+    const int tt = (int)(((long long)t_max + 64LL * ng * pack - 1) / (64LL * ng * pack)) * 64;
+    if (ng > 1 && tt < 256) break;
+    const long long rounds = ((long long)n_s * n_qb * ng + sms - 1) / sms, cost = rounds * (tt + lmax - 1 + kCtaAps);
+    if (cost < best) {
+      best = cost;
+      tile = tt;
+    }
+  }
+  return tile;
+}
+
 // Host planning: kernel arguments, series list and chunk size for `budget` bytes per set.
 // form: -1 = the FP32 tree (k_tree_mbd), else the tensor-core form of k_tree_mma (0 split BF16 x3,
 // 1 BF16, 2 E4M3).
 void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *windows, int n_win,
                const std::vector<int> &dkm, int n_bl, int T, int n_dm, const int *win_off, int S_tot, size_t budget,
-               int form, TreeRun *r, int TT = kTreeTT) {
+               int form, TreeRun *r, int TT = 0) {
   const bool mma = form >= 0;
   frbx::TreeArgs &t = r->t;
   t = frbx::TreeArgs{};
@@ -795,7 +820,9 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
   t.q_lo = a.q_lo;
   t.q_len = a.q_len;
   t.tw = h->d_tree_tw;
-  t.TT = TT;
+  // long scans on the tensor cores take time tiles of 2 x kTreeTT APs: half the trailing APs
+  // each tile re-reads and half the per-CTA setup, while the grid still spans many waves
+  t.TT = TT > 0 ? TT : mma && T >= 8 * kTreeTT ? 2 * kTreeTT : kTreeTT;
   t.n_tt = (T + t.TT - 1) / t.TT;
   t.k_per_cta = 16;
   t.n_ktile = (T + t.k_per_cta - 1) / t.k_per_cta;
@@ -816,7 +843,6 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
     t.pack = nq == 1 ? 4 : nq == 2 ? 2 : 1;
     t.prow = 128 / t.pack;
     t.piece_bytes = t.tile_bytes / t.pack;
-    t.n_tg = (t.n_tt + t.pack - 1) / t.pack;
     const int cols = frbx::tree_mma_cols(h->Lm, h->N);
     t.n_qb = (h->Lm + cols - 1) / cols;
     t.log2Lm = a.log2Lm;
@@ -845,6 +871,14 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
   const size_t per = sizeof(float2) * t.y_series + sc_per + anc_per;
   const size_t all = std::max<size_t>(r->ser.size(), 1);
   r->chunk = t.fused ? all : std::max<size_t>(1, std::min(all, budget / per));
+  if (mma) {
+    if (TT <= 0 && t.pack > 1 && !r->ser.empty()) {
+      const int t_max = T - *std::min_element(dkm.begin(), dkm.end());
+      t.TT = packed_time_tile(t_max, t.pack, (int)std::min(r->chunk, r->ser.size()), t.n_qb, 1 << nlev);
+      t.n_tt = (T + t.TT - 1) / t.TT;
+    }
+    t.n_tg = (t.n_tt + t.pack - 1) / t.pack;
+  }
   r->sc_off = (sizeof(float2) * t.y_series * r->chunk + 255) & ~(size_t)255;
   r->y_bytes = r->sc_off + ((sc_per * r->chunk + 255) & ~(size_t)255);
   r->a_bytes = (anc_per * r->chunk + 255) & ~(size_t)255;
@@ -942,11 +976,8 @@ int run_fit_tree(frbx_handle *h, const FitArgs &a, int nlev, int form, const int
     FRBX_CK(h, ensure(h, h->errflag, sizeof(int)));
     FRBX_CK(h, cudaMemsetAsync(h->errflag.p, 0, sizeof(int), st));
   }
-  // long scans on the tensor cores take time tiles of 2 x kTreeTT APs: half the trailing APs
-  // each tile re-reads and half the per-CTA setup, while the grid still spans many waves
-  const int TT = mma && T >= 8 * kTreeTT ? 2 * kTreeTT : kTreeTT;
   TreeRun r;
-  plan_tree(h, a, nlev, windows, n_win, dkm, n_bl, T, n_dm, d_tab + frbx::kMaxWin, S_tot, budget, form, &r, TT);
+  plan_tree(h, a, nlev, windows, n_win, dkm, n_bl, T, n_dm, d_tab + frbx::kMaxWin, S_tot, budget, form, &r);
   int rc = tree_prepare(h);
   if (rc) return rc;
   const size_t ser_bytes = (sizeof(int2) * std::max<size_t>(r.ser.size(), 1) + 255) & ~(size_t)255;
