@@ -3,8 +3,9 @@
 // (step d), the DM merge of the coarse DM search (Sec. 5.3) and cross-matching of
 // baselines.  Sequential and O(events x window length): each insertion asks "which
 // is the first group (in creation order) holding a member whose [k0, k0 + l) overlaps
-// mine", answered from a per-AP array of the smallest group id covering that AP.  Series are
-// independent until cross-matching, so large event lists are split across host threads.
+// mine", answered from a per-AP array of the smallest group id covering that AP.  Steps b to d of
+// one (series, DM trial) depend on its own events only, so event lists are split there
+// across host threads; the DM merge and cross-matching see the pulses of all, which are few.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -45,153 +46,160 @@ struct Grouper {
   }
 };
 
+// cos and sin of 2 pi q / Lm for every MBD cell, evaluated as for a single one
+struct CircleTable {
+  std::vector<double> th, c, s;
+  explicit CircleTable(int Lm) : th((size_t)std::max(Lm, 0)), c(th.size()), s(th.size()) {
+    for (size_t q = 0; q < th.size(); ++q) {
+      th[q] = (kTwoPi * (double)q) / (double)Lm;
+      c[q] = std::cos(th[q]);
+      s[q] = std::sin(th[q]);
+    }
+  }
+};
+
 // Step c: circular mean of the MBD over the group (period t_ambig; angle 2 pi q / Lm) and
 // removal of members at or beyond a quarter period from it.
-void mbd_filter(std::vector<const frbx_event *> *grp, int Lm) {
+void mbd_filter(std::vector<const frbx_event *> *grp, const CircleTable &t) {
   double sc = 0.0, ss = 0.0;
   for (const frbx_event *e : *grp) {
-    const double th = (kTwoPi * (double)e->mbd_idx) / (double)Lm;
-    sc += std::cos(th);
-    ss += std::sin(th);
+    sc += t.c[e->mbd_idx];
+    ss += t.s[e->mbd_idx];
   }
   const double mu = std::atan2(ss, sc);
-  std::vector<const frbx_event *> keep;
-  keep.reserve(grp->size());
+  size_t n = 0;
   for (const frbx_event *e : *grp) {
-    const double th = (kTwoPi * (double)e->mbd_idx) / (double)Lm;
-    if (std::fabs(std::remainder(th - mu, kTwoPi)) < M_PI / 2) keep.push_back(e);
+    // remainder(x, 2 pi) of x in [-pi, 3 pi): x or x - 2 pi, which is exact from pi on (Sterbenz)
+    const double x = t.th[e->mbd_idx] - mu, r = x > M_PI ? x - kTwoPi : x;
+    if (std::fabs(r) < M_PI / 2) (*grp)[n++] = e;
   }
-  grp->swap(keep);
+  grp->resize(n);
 }
 
-// Series [s_lo, s_hi) whose events are ev[0, n_ev) (sorted by series, DM trial, window, k0).
-void extract_range(const ExtractConfig &cfg, const frbx_event *ev, int64_t n_ev, int s_lo, int s_hi,
-                   bool use_mbd, std::vector<Pulse> *pre_merge, std::vector<Pulse> *merged) {
+// Steps b to d of the (series, DM trial)s whose events are ev[0, n_ev), sorted by series, DM trial,
+// window and k0: their pulses, in that order and, within one, in discovery order.
+void extract_events(const ExtractConfig &cfg, const CircleTable &circle, const frbx_event *ev, int64_t n_ev, bool use_mbd,
+                    std::vector<Pulse> *out) {
   // window visiting order: longest first (step b)
   std::vector<int> order(cfg.n_win);
   for (int w = 0; w < cfg.n_win; ++w) order[w] = w;
   std::stable_sort(order.begin(), order.end(),
                    [&](int x, int y) { return cfg.win_len[x] > cfg.win_len[y]; });
-  Grouper gp(cfg.T), gm(cfg.T);
-  int64_t pos = 0;
-  std::vector<std::vector<const frbx_event *>> groups;
+  Grouper gp(cfg.T);
+  std::vector<std::vector<const frbx_event *>> groups;  // the first n_groups are in use
   std::vector<std::pair<int64_t, int64_t>> wr(cfg.n_win);
-  for (int s = s_lo; s < s_hi; ++s) {
-    std::vector<Pulse> series_pulses;  // DM ascending, discovery order
-    for (int d = 0; d < cfg.n_dm; ++d) {
-      // the events of (s, d) are contiguous and ordered by window then k0
-      for (int w = 0; w < cfg.n_win; ++w) wr[w] = {0, 0};
-      while (pos < n_ev && ev[pos].series == s && ev[pos].dm_idx == d) {
-        const int w = ev[pos].win_idx;
-        int64_t e = pos;
-        while (e < n_ev && ev[e].series == s && ev[e].dm_idx == d && ev[e].win_idx == w) ++e;
-        wr[w] = {pos, e};
-        pos = e;
-      }
-      gp.reset();
-      groups.clear();
-      for (int w : order) {
-        for (int64_t i = wr[w].first; i < wr[w].second; ++i) {
-          const int g = gp.insert(ev[i].k0, cfg.win_len[w]);
-          if (g == (int)groups.size()) groups.emplace_back();
-          groups[(size_t)g].push_back(&ev[i]);
+  for (int64_t pos = 0; pos < n_ev;) {
+    const int s = ev[pos].series, d = ev[pos].dm_idx;
+    for (int w = 0; w < cfg.n_win; ++w) wr[w] = {0, 0};
+    while (pos < n_ev && ev[pos].series == s && ev[pos].dm_idx == d) {
+      const int w = ev[pos].win_idx;
+      int64_t e = pos;
+      while (e < n_ev && ev[e].series == s && ev[e].dm_idx == d && ev[e].win_idx == w) ++e;
+      wr[w] = {pos, e};
+      pos = e;
+    }
+    gp.reset();
+    size_t n_groups = 0;
+    for (int w : order) {
+      for (int64_t i = wr[w].first; i < wr[w].second; ++i) {
+        const size_t g = (size_t)gp.insert(ev[i].k0, cfg.win_len[w]);
+        if (g == n_groups) {
+          if (n_groups == groups.size()) groups.emplace_back();
+          groups[n_groups++].clear();
         }
-      }
-      for (auto &grp : groups) {
-        if (use_mbd) mbd_filter(&grp, cfg.Lm);
-        if (grp.empty()) continue;
-        // step d: distinct windows, best member (first inserted on ties)
-        int wins[kMaxWin];
-        int nw = 0;
-        for (const frbx_event *e : grp) {
-          bool seen = false;
-          for (int k = 0; k < nw; ++k) seen |= cfg.win_len[wins[k]] == cfg.win_len[e->win_idx];
-          if (!seen) wins[nw++] = e->win_idx;
-        }
-        if (nw < cfg.nwin_min) continue;
-        const frbx_event *best = grp[0];
-        for (const frbx_event *e : grp)
-          if (e->pnorm > best->pnorm) best = e;
-        Pulse p;
-        p.series = s;
-        p.d = d;
-        p.w = best->win_idx;
-        p.l = cfg.win_len[best->win_idx];
-        p.k0 = best->k0;
-        p.m = best->sbd_idx;
-        p.q = best->mbd_idx;
-        p.n_win = nw;
-        p.group = -1;
-        p.amp = best->amp;
-        p.p = best->pnorm;
-        series_pulses.push_back(p);
-        if (pre_merge) pre_merge->push_back(p);
+        groups[g].push_back(&ev[i]);
       }
     }
-    // Sec. 5.3: one pulse per overlap group across DM trials, the one of highest power
-    gm.reset();
-    std::vector<int> best_of;
-    for (size_t i = 0; i < series_pulses.size(); ++i) {
-      const int g = gm.insert(series_pulses[i].k0, series_pulses[i].l);
-      if (g == (int)best_of.size()) {
-        best_of.push_back((int)i);
-      } else if (series_pulses[i].p > series_pulses[(size_t)best_of[(size_t)g]].p) {
-        best_of[(size_t)g] = (int)i;
+    for (size_t gi = 0; gi < n_groups; ++gi) {
+      auto &grp = groups[gi];
+      if ((int)grp.size() < cfg.nwin_min) continue;  // fewer members than windows asked for
+      if (use_mbd) mbd_filter(&grp, circle);
+      if (grp.empty()) continue;
+      // step d: distinct windows (their lengths are distinct), best member (first inserted on ties)
+      unsigned seen = 0u;
+      const frbx_event *best = grp[0];
+      for (const frbx_event *e : grp) {
+        seen |= 1u << e->win_idx;
+        if (e->pnorm > best->pnorm) best = e;
       }
+      const int nw = __builtin_popcount(seen);
+      if (nw < cfg.nwin_min) continue;
+      Pulse p;
+      p.series = s;
+      p.d = d;
+      p.w = best->win_idx;
+      p.l = cfg.win_len[best->win_idx];
+      p.k0 = best->k0;
+      p.m = best->sbd_idx;
+      p.q = best->mbd_idx;
+      p.n_win = nw;
+      p.group = -1;
+      p.amp = best->amp;
+      p.p = best->pnorm;
+      out->push_back(p);
     }
-    for (int i : best_of) merged->push_back(series_pulses[(size_t)i]);
   }
 }
 
+// Sec. 5.3: per series, one pulse per overlap group across DM trials, the one of highest power.
+// pulses: sorted by series, DM trials ascending.
+void merge_dm(const ExtractConfig &cfg, const std::vector<Pulse> &pulses, std::vector<Pulse> *merged) {
+  Grouper gm(cfg.T);
+  std::vector<size_t> best_of;
+  for (size_t i = 0; i < pulses.size();) {
+    const int s = pulses[i].series;
+    gm.reset();
+    best_of.clear();
+    for (; i < pulses.size() && pulses[i].series == s; ++i) {
+      const size_t g = (size_t)gm.insert(pulses[i].k0, pulses[i].l);
+      if (g == best_of.size()) best_of.push_back(i);
+      else if (pulses[i].p > pulses[best_of[g]].p) best_of[g] = i;
+    }
+    for (size_t k : best_of) merged->push_back(pulses[k]);
+  }
+}
+
+// Events per host thread: a thread costs about 20 us to start, an event about 50 ns.
+constexpr int64_t kEventsPerThread = 2000;
+
 }  // namespace
 
-// The steps above depend only on one series' own events (steps b-d per DM trial, then the DM
-// merge of that series), so contiguous runs of series go to host threads, balanced by event
-// count, and their pulses are concatenated in series order: the same output as one pass.
+// Contiguous runs of (series, DM trial)s go to host threads, balanced by event count, the last one to
+// the calling thread, and their pulses are concatenated in order: the same output as one pass.
 void extract_pulses(const ExtractConfig &cfg, const frbx_event *ev, int64_t n_ev, int n_series,
                     bool use_mbd, std::vector<Pulse> *pre_merge, std::vector<Pulse> *merged) {
+  (void)n_series;
+  const CircleTable circle(use_mbd ? cfg.Lm : 0);
   const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
-  int n_th = n_ev < 50000 ? 1 : std::min({n_series, hw, 32});
-  for (int64_t i = 1; i < n_ev && n_th > 1; ++i)  // split points need events sorted by series
-    if (ev[i].series < ev[i - 1].series) n_th = 1;
-  if (n_th <= 1) {
-    extract_range(cfg, ev, n_ev, 0, n_series, use_mbd, pre_merge, merged);
-    return;
-  }
-  // first event of series s (events are sorted by series)
-  auto first_of = [&](int s) -> int64_t {
-    return std::lower_bound(ev, ev + n_ev, s, [](const frbx_event &e, int v) { return e.series < v; }) - ev;
-  };
-  // series cut points: part t ends at the first series whose first event reaches (t + 1) n_ev / n_th
-  std::vector<int> cut(n_th + 1, n_series);
+  const int n_th = (int)std::max<int64_t>(1, std::min<int64_t>({n_ev / kEventsPerThread, (int64_t)hw, (int64_t)32}));
+  // part t starts at the first event of a (series, DM trial) at or after t n_ev / n_th
+  std::vector<int64_t> cut((size_t)n_th + 1, n_ev);
   cut[0] = 0;
   for (int t = 1; t < n_th; ++t) {
-    const int64_t target = n_ev * t / n_th;
-    int s = cut[t - 1];
-    while (s < n_series && first_of(s) < target) ++s;
-    cut[t] = s;
+    int64_t i = std::max(cut[(size_t)t - 1], n_ev * t / n_th);
+    while (i > 0 && i < n_ev && ev[i].series == ev[i - 1].series && ev[i].dm_idx == ev[i - 1].dm_idx) ++i;
+    cut[(size_t)t] = i;
   }
-  std::vector<std::vector<Pulse>> pre_part(n_th), merged_part(n_th);
-  std::vector<std::thread> th;
-  th.reserve(n_th);
-  auto part = [&](int t) {
-    const int64_t e0 = first_of(cut[t]), e1 = first_of(cut[t + 1]);
-    extract_range(cfg, ev + e0, e1 - e0, cut[t], cut[t + 1], use_mbd, pre_merge ? &pre_part[t] : nullptr,
-                  &merged_part[t]);
+  std::vector<std::vector<Pulse>> part((size_t)n_th);
+  auto run = [&](int t) {
+    const int64_t e0 = cut[(size_t)t], e1 = cut[(size_t)t + 1];
+    if (e0 < e1) extract_events(cfg, circle, ev + e0, e1 - e0, use_mbd, &part[(size_t)t]);
   };
-  for (int t = 0; t < n_th; ++t) {
-    if (cut[t] >= cut[t + 1]) continue;
+  std::vector<std::thread> th;
+  th.reserve((size_t)n_th);
+  for (int t = 0; t + 1 < n_th; ++t) {
     try {
-      th.emplace_back(part, t);
+      th.emplace_back(run, t);
     } catch (...) {  // no thread to be had: this part runs here (no exception crosses the C ABI)
-      part(t);
+      run(t);
     }
   }
+  run(n_th - 1);
   for (auto &x : th) x.join();
-  for (int t = 0; t < n_th; ++t) {
-    if (pre_merge) pre_merge->insert(pre_merge->end(), pre_part[t].begin(), pre_part[t].end());
-    merged->insert(merged->end(), merged_part[t].begin(), merged_part[t].end());
-  }
+  std::vector<Pulse> all = std::move(part[0]);
+  for (int t = 1; t < n_th; ++t) all.insert(all.end(), part[(size_t)t].begin(), part[(size_t)t].end());
+  merge_dm(cfg, all, merged);
+  if (pre_merge) pre_merge->insert(pre_merge->end(), all.begin(), all.end());
 }
 
 void cross_match(int T, std::vector<Pulse> *merged, int n_bl, std::vector<GroupOut> *groups) {
