@@ -157,17 +157,42 @@ __device__ __forceinline__ bool tile_segment(const FitArgs &a, bool list, int i,
 __device__ __forceinline__ void gather_segment(const FitArgs &a, const ItemCtx &c, const Seg &s, float2 *X, int xs) {
   const int *dk = a.dk + (size_t)s.d * a.C;
   const size_t base = (size_t)s.bl * c.T + s.k0;
-  for (int p = threadIdx.x; p < a.C; p += blockDim.x) {
-    const float2 *src = c.vis + (base + __ldg(dk + p)) * a.C + p;
-    float2 acc = make_float2(0.f, 0.f);
-#pragma unroll 4
-    for (int i = 0; i < s.l; ++i) {
-      const float2 v = __ldg(src + (size_t)i * a.C);
-      acc.x += v.x;
-      acc.y += v.y;
+  // kGatherPts points of a thread side by side, kGatherAps APs of each loaded before they are added (in
+  // AP order): 16 loads in flight, where one point at a time waited for every fourth AP (20000 segments of
+  // 1 to 32 APs: 2.84 -> 2.44 ms)
+  constexpr int kGatherPts = 4, kGatherAps = 4;
+  for (int p0 = threadIdx.x; p0 < a.C; p0 += blockDim.x * kGatherPts) {
+    const float2 *src[kGatherPts];
+    float2 acc[kGatherPts];
+#pragma unroll
+    for (int q = 0; q < kGatherPts; ++q) {
+      const int p = min(p0 + q * (int)blockDim.x, a.C - 1);  // past the end: the last point again, not stored
+      src[q] = c.vis + (base + __ldg(dk + p)) * a.C + p;
+      acc[q] = make_float2(0.f, 0.f);
     }
-    const int n = p / a.J, j = p - n * a.J;
-    X[n * xs + j] = cmul(acc, __ldg(a.wrot + p));
+    for (int i = 0; i < s.l; i += kGatherAps) {
+      float2 v[kGatherPts][kGatherAps];
+#pragma unroll
+      for (int r = 0; r < kGatherAps; ++r)
+#pragma unroll
+        for (int q = 0; q < kGatherPts; ++q) v[q][r] = i + r < s.l ? __ldg(src[q] + (size_t)(i + r) * a.C) : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int r = 0; r < kGatherAps; ++r)
+#pragma unroll
+        for (int q = 0; q < kGatherPts; ++q)
+          if (i + r < s.l) {
+            acc[q].x += v[q][r].x;
+            acc[q].y += v[q][r].y;
+          }
+    }
+#pragma unroll
+    for (int q = 0; q < kGatherPts; ++q) {
+      const int p = p0 + q * (int)blockDim.x;
+      if (p < a.C) {
+        const int n = p / a.J, j = p - n * a.J;
+        X[n * xs + j] = cmul(acc[q], __ldg(a.wrot + p));
+      }
+    }
   }
 }
 

@@ -132,12 +132,16 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads)
       fft32_dif(A);
       unsigned key = 0u;
 #pragma unroll
-      for (int q2 = 0; q2 < 32; ++q2) {
-        const float2 v = A[bitrev5(q2)];
-        const float p = fmaf(v.x, v.x, v.y * v.y);
-        unsigned k = (__float_as_uint(p) & ~63u) | (unsigned)(32 - q2);
-        if (!kFull && (((q1 + PM * q2) - a.q_lo) & (Lm - 1)) >= a.q_len) k = 0u;
-        key = max(key, k);
+      for (int q2 = 0; q2 < 32; q2 += 2) {
+        unsigned k[2];
+#pragma unroll
+        for (int z = 0; z < 2; ++z) {
+          const float2 v = A[bitrev5(q2 + z)];
+          const float p = fmaf(v.x, v.x, v.y * v.y);
+          k[z] = (__float_as_uint(p) & ~63u) | (unsigned)(32 - q2 - z);
+          if (!kFull && (((q1 + PM * (q2 + z)) - a.q_lo) & (Lm - 1)) >= a.q_len) k[z] = 0u;
+        }
+        key = __vimax3_u32(key, k[0], k[1]);
       }
       if (key != 0u) better(bp, bi, __uint_as_float(key & ~63u), m * Lm + q1 + PM * (32 - (int)(key & 63u)));
     }

@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kThreads16, 3)
     }
 #pragma unroll
     for (int r = kSlots16; r < 16; ++r) g[r] = make_float2(0.f, 0.f);
-    fft16_dif(g);
+    fft16_dif<false>(g);
   };
 
   float2 ga[16], gb[16], h2[16];  // G_1 of two consecutive APs, G_2 of the last odd AP
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(kThreads16, 3)
 #pragma unroll
         for (int j2 = 0; j2 < 32; ++j2) A[j2] = cfma(A[j2], xr[j1 * 32 + j2], wr[j1 * 32 + j2]);
       }
-      fft32_dif(A);
+      fft32_dif<false>(A);
 #pragma unroll
       for (int i = 0; i < 32; ++i) yw[2 * kPS * bitrev5(i)] = A[i];
     }
