@@ -838,9 +838,9 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
     t.w_bytes = frbx::tree_mma_w_bytes(form, h->Lm, h->N);
     // delay windows: rotate the SBD rows so the searched ones come first (in groups of 8)
     t.rot = r->full ? 0 : (a.m_lo & ~7);
-    // rows searched after the rotation: [m_lo mod 8, m_lo mod 8 + m_len) in 32-row quarters
-    const int nq = r->full ? 4 : ((a.m_lo & 7) + a.m_len + 31) / 32;
-    t.pack = nq == 1 ? 4 : nq == 2 ? 2 : 1;
+    // rows searched after the rotation: [m_lo mod 8, m_lo mod 8 + m_len)
+    const int rows = r->full ? h->Ls : (a.m_lo & 7) + a.m_len;
+    t.pack = rows <= 16 ? 8 : rows <= 32 ? 4 : rows <= 64 ? 2 : 1;
     t.prow = 128 / t.pack;
     t.piece_bytes = t.tile_bytes / t.pack;
     const int cols = frbx::tree_mma_cols(h->Lm, h->N);

@@ -42,9 +42,10 @@
 // tile row r = (m - rot) mod Ls, so the searched rows sit in the first row quarters: warps whose
 // rows are all outside the SBD window only release their slots, cells outside the windows are
 // masked, and CTAs whose 32 q lie outside the MBD window exit at once.  When the searched rows
-// fit the first 32 (or 64) tile rows, the SBD pass keeps only those rows of each AP, and one CTA
-// stacks the pieces of four (or two) consecutive time tiles into its 128-row A operand: each
-// row quarter (pair) of warps walks its own time tile, so no epilogue warp idles.
+// fit the first 16, 32 or 64 tile rows, the SBD pass keeps only those rows of each AP, and one CTA
+// stacks the pieces of eight, four or two consecutive time tiles into its 128-row A operand: each
+// half of a row quarter's lanes, row quarter or pair of them walks its own time tile, so no epilogue
+// lane idles.
 // Every wait is bounded: on timeout the kernel records FRBX_ETIMEOUT, drains and frees its
 // tensor memory.
 #include <cuda_bf16.h>
@@ -408,12 +409,15 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
     const int quarter = warp & 3, part = warp >> 2;
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
     const uint32_t c_re = (uint32_t)(kQ * part), c_im = (uint32_t)(kNQ + kQ * part);
-    // this warp's time tile (its piece of the packed operand) and its first AP and AP count
-    const int qpp = 4 / pack, my_p = quarter / qpp;
-    const int kb_me = tile_kb(my_p), n_me = tile_n(my_p);
+    // this lane's time tile (its piece of the packed operand) and its first AP and AP count; the warp
+    // walks n_me APs, those of its first tile (with eight pieces a warp holds two, 16 lanes each, the
+    // second of them no longer)
+    const bool split = !kFull && pack == 8;
+    const int qpp = split ? 1 : 4 / pack, my_p = split ? 2 * quarter + (lane >> 4) : quarter / qpp;
+    const int kb_me = tile_kb(my_p), n_mine = tile_n(my_p), n_me = split ? tile_n(2 * quarter) : n_mine;
     // this lane's SBD row m (row (quarter mod qpp) 32 + lane of its piece, rotated by t.rot) and
     // its first cell
-    const int m_row = ((quarter % qpp) * 32 + lane + t.rot) & (t.Ls - 1);
+    const int m_row = (split ? (lane & 15) + t.rot : (quarter % qpp) * 32 + lane + t.rot) & (t.Ls - 1);
     const unsigned idx_base = (unsigned)(m_row * t.Lm + qb * kNQ + kQ * part);
     // delay windows: the lane's row is searched, and which of its kQ cells
     const bool row_on = kFull || (((m_row - t.m_lo) & (t.Ls - 1)) < t.m_len);
@@ -497,22 +501,29 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
     // starting before the tile is never issued)
     unsigned long long *const base0 = keys + woff[0] + kb_me, *const base1 = keys + woff[1] + kb_me,
                               *const base2 = keys + woff[2] + (kb_me >> 1);
+    // (the delay-window form has no registers to spare for them: slots, added to keys at each merge)
+    const int o0 = woff[0] + kb_me, o1 = woff[1] + kb_me, o2 = woff[2] + (kb_me >> 1);
     auto merge = [&](const int e, const int i0, const unsigned tkey, const bool on) {
-      const unsigned wmax = __reduce_max_sync(0xffffffffu, tkey);
+      unsigned wmax = __reduce_max_sync(0xffffffffu, !kFull && split && lane >= 16 ? 0u : tkey);
+      if (!kFull && split) {  // each tile's 16 lanes by themselves
+        const unsigned hi = __reduce_max_sync(0xffffffffu, lane >= 16 ? tkey : 0u);
+        if (lane >= 16) wmax = hi;
+      }
       // every lane forms the merge; the lanes holding the maximum issue it (predicated, no branch)
       const unsigned idx = idx_base + (31u - (wmax & 63u));
       // slot of the segment: windows of 2^e APs start every 2^(e-1) APs (every AP for e = 0)
-      unsigned long long *dst = e == 0   ? base0 + i0
+      unsigned long long *dst = e > 2    ? keys + woff[e] + ((kb_me + i0) >> (e - 1))
+                                : !kFull ? keys + (e == 0 ? o0 + i0 : e == 1 ? o1 + i0 : o2 + (i0 >> 1))
+                                : e == 0 ? base0 + i0
                                 : e == 1 ? base1 + i0
-                                : e == 2 ? base2 + (i0 >> 1)
-                                         : keys + woff[e] + ((kb_me + i0) >> (e - 1));
+                                         : base2 + (i0 >> 1);
       const unsigned long long kv = ((unsigned long long)(wmax & ~63u) << 32) | (unsigned long long)(~idx);
       asm volatile("{\n .reg .pred p;\n setp.eq.u32 p, %2, %3;\n setp.ne.and.u32 p, %3, 0, p;\n"
                    " setp.ne.and.u32 p, %4, 0, p;\n @p red.relaxed.gpu.global.max.u64 [%0], %1;\n}\n"
                    ::"l"(dst), "l"(kv), "r"(tkey), "r"(wmax), "r"((unsigned)on) : "memory");
     };
-    auto emit = [&](const int e, const int i0, const uint64_t(&gre)[kP], const uint64_t(&gim)[kP]) {
-      merge(e, i0, seg_top(gre, gim), true);
+    auto emit = [&](const int e, const int i0, const uint64_t(&gre)[kP], const uint64_t(&gim)[kP], const bool on) {
+      merge(e, i0, seg_top(gre, gim), on);
     };
     // One AP: cur receives G_1(k); pre holds G_1(k - 1).  odd: k is odd (counted from the tile's
     // first AP, a multiple of 64), so it closes a window of 4 APs: the level-1 sum
@@ -533,7 +544,7 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
       tm_ld(cur + c_im, rim);
 
       float inv_s = 1.f;  // E4M3 form: the AP's A was scaled by s, a power of two
-      if constexpr (kForm == kFormFp8) inv_s = __ldg(t.ascale + (size_t)s * t.T + kb_me + i);
+      if constexpr (kForm == kFormFp8) inv_s = __ldg(t.ascale + (size_t)s * t.T + min(kb_me + i, t.T - 1));
       // levels whose window ends at AP kb_me + i, and which of them emit a segment of this time
       // tile (uniform across the warp; kb_me is a multiple of 2^kTmMaxLev, so i's low bits
       // decide)
@@ -548,6 +559,7 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
           if (i0 < 0 || i0 >= t.TT) em &= ~(1u << e);
         }
       }
+      if (!kFull && i >= n_mine) em = 0u;  // the second tile of the warp has ended
       tm_wait_ld();
       tm_take(rre, cre);
       tm_take(rim, cim);
@@ -657,7 +669,7 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
           aim[p] = add2(aim[p], oim[p]);
         }
         if (in_tmem) tm_wait_st();
-        if ((em >> e) & 1u) emit(e, i - (1 << e) + 1, are, aim);
+        if (__any_sync(0xffffffffu, (em >> e) & 1u)) emit(e, i - (1 << e) + 1, are, aim, (em >> e) & 1u);
       }
       return true;
     };
@@ -768,7 +780,7 @@ cudaError_t launch_tree_mma(const TreeArgs &t, bool full, cudaStream_t st, int64
       t.w_bytes != tm_w_bytes(t.form, t.N, parts) || t.tile_bytes != tm_tile_bytes(t.form, t.N) ||
       t.n_qb != (t.Lm + cols - 1) / cols ||
       (t.form == kFormFp8 && (!t.ascale || t.k8_steps != (2 * t.N + 31) / 32)) || (full && t.rot != 0) ||
-      (t.rot & 7) != 0 || !(t.pack == 1 || t.pack == 2 || t.pack == 4) || (full && t.pack != 1) ||
+      (t.rot & 7) != 0 || !(t.pack == 1 || t.pack == 2 || t.pack == 4 || t.pack == 8) || (full && t.pack != 1) ||
       t.prow * t.pack != tc::kRows || t.piece_bytes * t.pack != t.tile_bytes || t.n_tg * t.pack < t.n_tt ||
       t.TT % (1 << kTmMaxLev) != 0)
     return cudaErrorInvalidValue;
