@@ -226,7 +226,9 @@ void set_tree16_constants();
 // kernels_misc.cu
 cudaError_t launch_shift_table(const double *f, int C, double fref, const double *dm, int n_dm,
                                double t_ap, int *dk, int *dk_max, cudaStream_t st,
-                               int64_t *launches);
+                               int64_t *launches);  // dk_max may be null
+// one shift of Eq. 1-2 on the host, by the operations of the device table
+int shift_of(double f, double inv_fref2, double dm, double t_ap);
 
 struct StatsArgs {
   const frbx_seg *series;  // [n_bl][n_dm][S_tot]
@@ -314,6 +316,7 @@ struct frbx_handle {
   };
   frbx_limits lim{};          // frbx_set_limits (all zero = defaults)
   size_t scratch_total = 0;   // bytes held by the Bufs below
-  Buf vis, dk, dk_max, series, pnorm, stats, counts, offsets, events, small, seglist, masks, hits, errflag, refine, calib,
+  const int *dk_max = nullptr;  // [n_dm] in dm_in, of the last shift table
+  Buf vis, dk, dm_in, series, pnorm, stats, counts, offsets, events, small, seglist, masks, hits, errflag, refine, calib,
       ytree;
 };

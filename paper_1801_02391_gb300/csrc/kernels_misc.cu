@@ -1,6 +1,7 @@
 // Dispersion shift table (Eq. 1-2) and the normalisation / threshold stage (Eq. 6,
 // Sec. 2.4.1 step a) for baselines and for baseline combinations (Sec. 2.4.2 step b).
 #include <cfloat>
+#include <cmath>
 
 #include "frbx_internal.h"
 
@@ -39,6 +40,11 @@ __global__ void k_row_max(const int *__restrict__ dk, int C, int *__restrict__ o
   }
 }
 
+int shift_of(double f, double inv_fref2, double dm, double t_ap) {
+  const double b = 1.0 / (f * f) - inv_fref2, dt = (4.15e6 * dm) * b;
+  return (int)std::floor(std::fmin(0.5 + dt / t_ap, 1.0e9));
+}
+
 cudaError_t launch_shift_table(const double *f, int C, double fref, const double *dm, int n_dm,
                                double t_ap, int *dk, int *dk_max, cudaStream_t st,
                                int64_t *launches) {
@@ -49,8 +55,10 @@ cudaError_t launch_shift_table(const double *f, int C, double fref, const double
   k_shift_table<<<(unsigned)((n + threads - 1) / threads), threads, 0, st>>>(f, C, inv_fref2, dm,
                                                                             n_dm, t_ap, dk);
   ++*launches;
-  k_row_max<<<n_dm, 256, 0, st>>>(dk, C, dk_max);
-  ++*launches;
+  if (dk_max) {
+    k_row_max<<<n_dm, 256, 0, st>>>(dk, C, dk_max);
+    ++*launches;
+  }
   return cudaGetLastError();
 }
 
