@@ -293,7 +293,7 @@ struct frbx_handle {
   float2 *d_tree_tw = nullptr;  // [16 s16][Lm/32][2] MBD twiddles of the window-tree fit
   int *d_tree_slot = nullptr;   // [N] channel slot of the window-tree fit
   int tree_s16 = 0;             // slots per residue class mod 16 (0: no window-tree fit)
-  cudaStream_t tree_st[2] = {nullptr, nullptr};  // window-tree fit: SBD passes, MBD passes
+  cudaStream_t tree_st[3] = {nullptr, nullptr, nullptr};  // window-tree fit: SBD passes, MBD passes of even and odd chunks
   cudaEvent_t tree_ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // start, SBD done x2, MBD done x2
   std::vector<cudaEvent_t> tree_kev;  // per window-tree chunk: SBD start / end, MBD start / end
   // host input of a search: the cube is copied one baseline after another on copy_st; vis_ev[b]
