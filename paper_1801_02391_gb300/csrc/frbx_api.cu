@@ -799,7 +799,7 @@ int packed_time_tile(int t_max, int pack, int n_s, int n_qb, int lmax) {
 // 1 BF16, 2 E4M3).
 void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *windows, int n_win,
                const std::vector<int> &dkm, int n_bl, int T, int n_dm, const int *win_off, int S_tot, size_t budget,
-               int form, TreeRun *r, int TT = 0) {
+               int form, TreeRun *r, int TT = 0, bool copying = false) {
   const bool mma = form >= 0;
   frbx::TreeArgs &t = r->t;
   t = frbx::TreeArgs{};
@@ -877,7 +877,10 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
   const size_t sc_per = form == 2 ? sizeof(float) * (size_t)T : 0;
   const size_t per = sizeof(float2) * t.y_series + sc_per + anc_per;
   const size_t all = std::max<size_t>(r->ser.size(), 1);
-  r->chunk = t.fused ? all : std::max<size_t>(1, std::min(all, budget / per));
+  // a cube still being copied from the host, one baseline after another: no chunk waits for more than
+  // one (a search of 2 baselines x 2411 APs from pinned memory 6.27 -> 6.11 ms)
+  const size_t most = copying && mma ? std::max<size_t>(1, all / (size_t)n_bl) : all;
+  r->chunk = t.fused ? all : std::max<size_t>(1, std::min(most, budget / per));
   if (mma) {
     if (TT <= 0 && t.pack > 1 && !r->ser.empty()) {
       const int t_max = T - *std::min_element(dkm.begin(), dkm.end());
@@ -990,7 +993,8 @@ int run_fit_tree(frbx_handle *h, const FitArgs &a, int nlev, int form, const int
     FRBX_CK(h, cudaMemsetAsync(h->errflag.p, 0, sizeof(int), st));
   }
   TreeRun r;
-  plan_tree(h, a, nlev, windows, n_win, dkm, n_bl, T, n_dm, d_tab + frbx::kMaxWin, S_tot, budget, form, &r);
+  plan_tree(h, a, nlev, windows, n_win, dkm, n_bl, T, n_dm, d_tab + frbx::kMaxWin, S_tot, budget, form, &r, 0,
+            copied != nullptr);
   int rc = tree_prepare(h);
   if (rc) return rc;
   const size_t ser_bytes = (sizeof(int2) * std::max<size_t>(r.ser.size(), 1) + 255) & ~(size_t)255;
