@@ -71,13 +71,18 @@ __device__ __forceinline__ void bulk_s2g(void *dst, const void *src, uint32_t by
 // spectrum, which bounds every |Re Y|, |Im Y|), 1 / s stored in t.ascale.  Tile row r holds SBD
 // row (r + t.rot) mod Ls (rotation for delay windows; 0 for the whole grid); with t.pack > 1
 // only the first t.prow rows of every K atom are stored (t.piece_bytes per AP).
-template <int kOut>
+// kRot: the rows are rotated; without it every store's offset is an immediate added to the thread's own
+// (the rotated row group is three instructions a value).  With the two-point reads below, a ninth of
+// the instructions: 192 series x 20000 APs 248.4 -> 246.8 ms, 96 x 9973 with a window 26.45 -> 26.21 ms.
+template <int kOut, bool kRot>
 __global__ void __launch_bounds__(kTreeThreads, 4)
     k_tree_sbd(const __grid_constant__ FitArgs a, const __grid_constant__ TreeArgs t) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ float red_l1[kTreeThreads / 32];
   const int N = a.N, Ls = a.Ls, PS = Ls >> 5, lps = __ffs(PS) - 1;
-  const int JP = a.J1 * 32, xs = JP + 1;
+  // even row strides: 16-byte reads of two points at once, whose 8 (or, of the twiddles, PS) rows per
+  // warp fall 16 bytes apart on the banks
+  const int JP = a.J1 * 32, xs = JP + 2;
   const int stage = kOut ? t.tile_bytes : (int)sizeof(float2) * Ls * N;  // one AP of output
   float2 *Ys = reinterpret_cast<float2 *>(smem);                        // [Ls][N] or the tiles
   unsigned char *Yb = smem;
@@ -99,7 +104,7 @@ __global__ void __launch_bounds__(kTreeThreads, 4)
   float4 *Yout = kOut ? reinterpret_cast<float4 *>(const_cast<unsigned char *>(t.Yt) + (size_t)s * t.yt_series)
                       : reinterpret_cast<float4 *>(t.Y + (size_t)s * t.y_series);
   const int row4 = stage / 16;  // float4 per AP
-  const int rot8 = t.rot >> 3;  // rotation in groups of 8 rows
+  const int rot8 = kRot ? t.rot >> 3 : 0;  // rotation in groups of 8 rows
   // this thread's points p = tid + blockDim i: channel n and point j stepped without a division
   const int dn = (int)blockDim.x / a.J, dj = (int)blockDim.x - dn * a.J;
   const int n0 = (int)threadIdx.x / a.J, j0 = (int)threadIdx.x - n0 * a.J;
@@ -177,7 +182,12 @@ __global__ void __launch_bounds__(kTreeThreads, 4)
       const float2 *wr = stw + m1 * xs;
       for (int j1 = 0; j1 < a.J1; ++j1) {
 #pragma unroll
-        for (int j2 = 0; j2 < 32; ++j2) A[j2] = cfma(A[j2], xr[j1 * 32 + j2], wr[j1 * 32 + j2]);
+        for (int j2 = 0; j2 < 32; j2 += 2) {
+          const float4 x = *reinterpret_cast<const float4 *>(xr + j1 * 32 + j2);
+          const float4 w = *reinterpret_cast<const float4 *>(wr + j1 * 32 + j2);
+          A[j2] = cfma(A[j2], make_float2(x.x, x.y), make_float2(w.x, w.y));
+          A[j2 + 1] = cfma(A[j2 + 1], make_float2(x.z, x.w), make_float2(w.z, w.w));
+        }
       }
       fft32_dif(A);
       if (kOut == 1 || kOut == 2) {
@@ -195,7 +205,7 @@ __global__ void __launch_bounds__(kTreeThreads, 4)
         }
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
-          const int b = bitrev5(i), row = (m1 + PS * b - t.rot) & (Ls - 1);
+          const int b = bitrev5(i), row = (m1 + PS * b - 8 * rot8) & (Ls - 1);
           const __nv_bfloat16 rh = __float2bfloat16_rn(A[i].x), ih = __float2bfloat16_rn(A[i].y);
           const uint32_t grp = (uint32_t)(((b >> 1) - rot8) & 15) * 1024u;
           const uint32_t orr = PS == 4 ? o_re[b & 1] + grp : tc::a_offset(row, n);
@@ -220,7 +230,7 @@ __global__ void __launch_bounds__(kTreeThreads, 4)
         }
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
-          const int b = bitrev5(i), row = (m1 + PS * b - t.rot) & (Ls - 1);
+          const int b = bitrev5(i), row = (m1 + PS * b - 8 * rot8) & (Ls - 1);
           const uint32_t grp = (uint32_t)(((b >> 1) - rot8) & 15) * 1024u;
           const uint32_t orr = PS == 4 ? o_re[b & 1] + grp : tc::a_offset8(row, n);
           const uint32_t oi = PS == 4 ? o_im[b & 1] + grp : tc::a_offset8(row, N + n);
@@ -484,7 +494,7 @@ bool tree_supported(int Ls, int Lm, int N, int J, int s16, const int *windows, i
   // the SBD pass holds one AP of output (Ls N complex, the same bytes as the split tiles of the
   // tensor-core form), the gathered points and its twiddles
   const int JP = (J + 31) / 32 * 32;
-  const size_t sbd = sizeof(float2) * ((size_t)Ls * N + (size_t)N * (JP + 1) + (size_t)(Ls / 32) * (JP + 1));
+  const size_t sbd = sizeof(float2) * ((size_t)Ls * N + (size_t)N * (JP + 2) + (size_t)(Ls / 32) * (JP + 2));
   return tree_smem_bytes(NS, PM, RB, *nlev) <= max_smem_optin() && sbd <= max_smem_optin();
 }
 
@@ -495,7 +505,7 @@ size_t tree_anchor_floats(int nlev) { return (size_t)tree_global_anchors(nlev) *
 size_t tree_sbd_smem(const FitArgs &a, const TreeArgs &t) {
   const int JP = a.J1 * 32;
   const size_t stage = t.mma ? (size_t)t.tile_bytes : sizeof(float2) * (size_t)a.Ls * a.N;
-  return stage + sizeof(float2) * ((size_t)a.N * (JP + 1) + (size_t)(a.Ls / 32) * (JP + 1));
+  return stage + sizeof(float2) * ((size_t)a.N * (JP + 2) + (size_t)(a.Ls / 32) * (JP + 2));
 }
 
 cudaError_t launch_tree_sbd(const FitArgs &a, const TreeArgs &t, cudaStream_t st, int64_t *launches) {
@@ -506,7 +516,9 @@ cudaError_t launch_tree_sbd(const FitArgs &a, const TreeArgs &t, cudaStream_t st
   if (!t.mma && t.rot != 0) return cudaErrorInvalidValue;
   if (t.mma && (t.pack < 1 || t.piece_bytes * t.pack != t.tile_bytes || t.prow * t.pack != tc::kRows))
     return cudaErrorInvalidValue;
-  auto kern = !t.mma ? k_tree_sbd<0> : t.form == 0 ? k_tree_sbd<1> : t.form == 1 ? k_tree_sbd<2> : k_tree_sbd<3>;
+  auto kern = !t.mma ? k_tree_sbd<0, false>
+              : t.rot ? (t.form == 0 ? k_tree_sbd<1, true> : t.form == 1 ? k_tree_sbd<2, true> : k_tree_sbd<3, true>)
+                      : (t.form == 0 ? k_tree_sbd<1, false> : t.form == 1 ? k_tree_sbd<2, false> : k_tree_sbd<3, false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)nb, kTreeThreads, smem, st>>>(a, t);
