@@ -64,6 +64,20 @@ __device__ __forceinline__ void fft32_dif(float2 (&a)[32]) {
   dif_stage<kPacked, 32, 2, 0>(a);
   dif_stage<kPacked, 32, 1, 0>(a);
 }
+// The same 16-point DFT as fft16_dif of inputs whose upper eight are zero (left unset): the first stage
+// only copies and turns.
+template <int K>
+__device__ __forceinline__ void low_bfly(float2 (&a)[16]) {
+  a[K + 8] = twiddle32<2 * K>(a[K]);
+  if constexpr (K + 1 < 8) low_bfly<K + 1>(a);
+}
+template <bool kPacked = true>
+__device__ __forceinline__ void fft16_dif_low(float2 (&a)[16]) {
+  low_bfly<0>(a);
+  dif_stage<kPacked, 16, 4, 0>(a);
+  dif_stage<kPacked, 16, 2, 0>(a);
+  dif_stage<kPacked, 16, 1, 0>(a);
+}
 // In-place 16-point DFT (forward, exp(-i)); output k holds frequency bitrev4(k).
 template <bool kPacked = true>
 __device__ __forceinline__ void fft16_dif(float2 (&a)[16]) {

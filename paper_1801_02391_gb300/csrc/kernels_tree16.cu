@@ -15,6 +15,7 @@
 // results are the same bits; segments' maxima are merged per warp by a 64-bit atomicMax.
 // The S-band search of 3 baselines x 101 DM trials x 4096 APs: both passes 13.0 -> 3.1 ms (the two-pass
 // form issued on few of its cycles: two serial device reads per AP, half of each CTA's threads idle).
+// Three-input maxima, a first FFT stage without its zeros and reads of two points: call 4.64 -> 4.55 ms.
 #include "fit_common.cuh"
 #include "fft32.cuh"
 
@@ -31,7 +32,7 @@ constexpr int kMaxLev16 = 6;  // windows up to 64 APs
 // SBD rows of a pair of slots: padded so that the pairs' rows fall on different banks
 __host__ __device__ constexpr int pair_stride(int Ls) { return Ls + 2; }
 __host__ __device__ inline size_t tree16_smem(int Ls, int N, int J1) {
-  const int aps = kThreads16 / Ls * kStep16, xs = J1 * 32 + 1;
+  const int aps = kThreads16 / Ls * kStep16, xs = J1 * 32 + 2;
   return sizeof(float4) * (size_t)aps * (kSlots16 / 2) * pair_stride(Ls) +
          sizeof(float2) * ((size_t)aps * N * xs + (size_t)(Ls / 32) * xs);
 }
@@ -45,7 +46,7 @@ __global__ void __launch_bounds__(kThreads16, 3)
   constexpr int Ls = 32 * kPS, kSub = kThreads16 / Ls, kAps = kSub * kStep16, kPairs = kSlots16 / 2;
   constexpr int kYAp = kPairs * pair_stride(Ls);  // float4 per AP
   extern __shared__ __align__(16) unsigned char smem[];
-  const int N = a.N, J = a.J, C = a.C, xs = a.J1 * 32 + 1;
+  const int N = a.N, J = a.J, C = a.C, xs = a.J1 * 32 + 2;  // even: two points a read, rows 16 bytes apart on the banks
   float4 *Y = reinterpret_cast<float4 *>(smem);           // [kAps][kPairs][Ls + 2] slots 2p, 2p + 1
   float2 *X = reinterpret_cast<float2 *>(Y + kAps * kYAp);  // [kAps][N][xs]
   float2 *stw = X + kAps * N * xs;                        // [kPS][xs]
@@ -127,17 +128,18 @@ __global__ void __launch_bounds__(kThreads16, 3)
   auto emit = [&](const int e, const int i, const float2(&g)[16]) {
     const int w = t.emit_w[e], i0 = i - (1 << e) + 1;
     if (w < 0 || i >= n_ap || i0 < 0 || i0 >= t.TT) return;  // uniform across the warp
-    unsigned key = 0u;
+    unsigned k[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
-      unsigned k = cell_key<kFull>(g[c], bitrev5(c) >> 1, 0, kmask);
-      if (!kFull) k = (cmask >> c) & 1u ? k : 0u;
-      key = max(key, k);
+      k[c] = cell_key<kFull>(g[c], bitrev5(c) >> 1, 0, kmask);
+      if (!kFull) k[c] = (cmask >> c) & 1u ? k[c] : 0u;
     }
+#pragma unroll
+    for (int c = 0; c < 5; ++c) k[c] = __vimax3_u32(k[c], k[c + 5], k[c + 10]);
+    const unsigned key = __vimax3_u32(__vimax3_u32(k[0], k[1], k[2]), __vimax3_u32(k[3], k[4], k[15]), 0u);
     const unsigned wmax = __reduce_max_sync(0xffffffffu, key);
-    const unsigned win = __ballot_sync(0xffffffffu, key == wmax);
     const unsigned pw = wmax & (kFull ? ~15u : ~63u);
-    if (lane == __ffs(win) - 1 && pw != 0u) {
+    if (key == wmax && pw != 0u) {  // tied lanes share the column; the merge keeps the lowest row
       const unsigned q = kFull ? 15u - (wmax & 15u) : (32u - (wmax & 63u)) >> 1;
       const unsigned idx = (unsigned)m * 16u + q;
       // windows of 2^e APs start every 2^(e-1) APs (every AP for e = 0)
@@ -153,9 +155,7 @@ __global__ void __launch_bounds__(kThreads16, 3)
       g[2 * p] = cfma(make_float2(0.f, 0.f), make_float2(y.x, y.y), unit);
       g[2 * p + 1] = cfma(make_float2(0.f, 0.f), make_float2(y.z, y.w), unit);
     }
-#pragma unroll
-    for (int r = kSlots16; r < 16; ++r) g[r] = make_float2(0.f, 0.f);
-    fft16_dif<false>(g);
+    fft16_dif_low<false>(g);
   };
 
   float2 ga[16], gb[16], h2[16];  // G_1 of two consecutive APs, G_2 of the last odd AP
@@ -172,7 +172,12 @@ __global__ void __launch_bounds__(kThreads16, 3)
       for (int i = 0; i < 32; ++i) A[i] = make_float2(0.f, 0.f);
       for (int j1 = 0; j1 < a.J1; ++j1) {
 #pragma unroll
-        for (int j2 = 0; j2 < 32; ++j2) A[j2] = cfma(A[j2], xr[j1 * 32 + j2], wr[j1 * 32 + j2]);
+        for (int j2 = 0; j2 < 32; j2 += 2) {
+          const float4 x = *reinterpret_cast<const float4 *>(xr + j1 * 32 + j2);
+          const float4 w = *reinterpret_cast<const float4 *>(wr + j1 * 32 + j2);
+          A[j2] = cfma(A[j2], make_float2(x.x, x.y), make_float2(w.x, w.y));
+          A[j2 + 1] = cfma(A[j2 + 1], make_float2(x.z, x.w), make_float2(w.z, w.w));
+        }
       }
       fft32_dif<false>(A);
 #pragma unroll
