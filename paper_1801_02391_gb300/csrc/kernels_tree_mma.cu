@@ -210,7 +210,9 @@ __device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint64_t ad, uint64_t 
 // ring (t.n_abuf deep), then the t.n_sanc deepest anchor levels as [level][column quads][128 rows]
 // float4.  kForm: the MBD product (above); kFull: the whole delay grid is searched (no windows, no row
 // rotation).
-template <int kParts, int kForm, bool kFull>
+// kOne: windows of one AP are searched; without them no AP's own maximum is formed, a sixth of the
+// epilogue's instructions (built for the default product; five scans with windows of 2 to 16 APs: 50.4 -> 46.7 ms).
+template <int kParts, int kForm, bool kFull, bool kOne>
 __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(const __grid_constant__ TreeArgs t) {
   using Sh = TmShape<kParts>;
   constexpr int kEpi = Sh::kEpi, kMmaWarp = kEpi, kLoadWarp = kEpi + 1, kNQ = Sh::kNQ, kCols = Sh::kCols;
@@ -584,8 +586,8 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
           are[p] = add2(pre[p], cre[p]);
           aim[p] = add2(pim[p], cim[p]);
         }
-        const unsigned top0 = seg_top(cre, cim), top1 = seg_top(are, aim);
-        merge(0, i, top0, (em & 1u) != 0u);
+        const unsigned top0 = kOne ? seg_top(cre, cim) : 0u, top1 = seg_top(are, aim);
+        if (kOne) merge(0, i, top0, (em & 1u) != 0u);
         merge(1, i - 1, top1, (em & 2u) != 0u);
         return true;
       }
@@ -602,8 +604,8 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
           are[p] = add2(ain_re[p], aout_re[p]);
           aim[p] = add2(ain_im[p], aout_im[p]);
         }
-        const unsigned top0 = seg_top(cre, cim), top1 = seg_top(aout_re, aout_im), top2 = seg_top(are, aim);
-        merge(0, i, top0, (em & 1u) != 0u);
+        const unsigned top0 = kOne ? seg_top(cre, cim) : 0u, top1 = seg_top(aout_re, aout_im), top2 = seg_top(are, aim);
+        if (kOne) merge(0, i, top0, (em & 1u) != 0u);
         merge(1, i - 1, top1, (em & 2u) != 0u);
         merge(2, i - 3, top2, ((em >> 2) & 1u) != 0u);
       } else {
@@ -618,8 +620,8 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
           are[p] = add2(pre[p], cre[p]);
           aim[p] = add2(pim[p], cim[p]);
         }
-        const unsigned top0 = seg_top(cre, cim), top1 = seg_top(are, aim);
-        merge(0, i, top0, (em & 1u) != 0u);
+        const unsigned top0 = kOne ? seg_top(cre, cim) : 0u, top1 = seg_top(are, aim);
+        if (kOne) merge(0, i, top0, (em & 1u) != 0u);
         merge(1, i - 1, top1, (em & 2u) != 0u);
         uint64_t ore[kP], oim[kP];
         tm_wait_ld();
@@ -747,10 +749,10 @@ bool tree_mma_fits(int form, int Lm, int N, int nlev) {
 int tree_mma_tile_bytes(int form, int N) { return tm_tile_bytes(form, N); }
 int tree_mma_w_bytes(int form, int Lm, int N) { return tm_w_bytes(form, N, tree_mma_cols(Lm, N) / kQ); }
 
-template <int kParts, int kForm, bool kFull>
+template <int kParts, int kForm, bool kFull, bool kOne = true>
 static cudaError_t launch_tm_one(const TreeArgs &u, unsigned nb, size_t smem, cudaStream_t st) {
   using Sh = TmShape<kParts>;
-  auto kern = k_tree_mma<kParts, kForm, kFull>;
+  auto kern = k_tree_mma<kParts, kForm, kFull, kOne>;
   // the register split inside the kernel assumes the launch allocation of kLaunchRegs per thread
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, kern);
@@ -764,6 +766,9 @@ static cudaError_t launch_tm_one(const TreeArgs &u, unsigned nb, size_t smem, cu
 
 template <int kParts>
 static cudaError_t launch_tm(const TreeArgs &u, bool full, unsigned g, size_t smem, cudaStream_t st) {
+  if (u.form == kFormSplit && u.emit_w[0] < 0)
+    return full ? launch_tm_one<kParts, kFormSplit, true, false>(u, g, smem, st)
+                : launch_tm_one<kParts, kFormSplit, false, false>(u, g, smem, st);
   switch (u.form * 2 + (full ? 1 : 0)) {
     case 0: return launch_tm_one<kParts, kFormSplit, false>(u, g, smem, st);
     case 1: return launch_tm_one<kParts, kFormSplit, true>(u, g, smem, st);
