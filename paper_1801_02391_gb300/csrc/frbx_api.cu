@@ -565,7 +565,9 @@ int run_shift_table(frbx_handle *h, const double *dm, int n_dm, std::vector<int>
   const double inv_fref2 = 1.0 / (h->f_ref * h->f_ref), f_low = *std::min_element(h->f.begin(), h->f.end());
   dk_max->resize((size_t)n_dm);
   for (int d = 0; d < n_dm; ++d) (*dk_max)[(size_t)d] = frbx::shift_of(f_low, inv_fref2, dm[d], h->t_ap);
-  std::vector<unsigned char> in(b_in);
+  // kept in the handle: the copy may still be reading it when this function returns
+  std::vector<unsigned char> &in = h->dm_host;
+  in.resize(b_in);
   std::memcpy(in.data(), dm, b_dm);
   std::memcpy(in.data() + b_dm, dk_max->data(), b_in - b_dm);
   FRBX_CK(h, cudaMemcpyAsync(h->dm_in.p, in.data(), b_in, cudaMemcpyHostToDevice, st));
@@ -1186,7 +1188,10 @@ static int fit_segments_impl(frbx_handle *h, const void *vis, int32_t vis_on_dev
         (long long)r[3] + dkm[(size_t)r[1]] + r[2] > T)
       return fail(h, FRBX_EINVAL, "segment row " + std::to_string(i) + " reads outside the cube");
   }
-  if (n_seg == 0) return FRBX_OK;
+  if (n_seg == 0) {  // the caller may release its cube: host input is still being copied
+    FRBX_CK(h, cudaStreamSynchronize(st));
+    return FRBX_OK;
+  }
   FRBX_CK(h, ensure(h, h->seglist, sizeof(int32_t) * 4 * (size_t)n_seg));
   FRBX_CK(h, ensure(h, h->series, sizeof(frbx_seg) * (size_t)n_seg));
   FRBX_CK(h, cudaMemcpyAsync(h->seglist.p, segs, sizeof(int32_t) * 4 * (size_t)n_seg, cudaMemcpyHostToDevice, st));

@@ -316,6 +316,7 @@ struct frbx_handle {
   };
   frbx_limits lim{};          // frbx_set_limits (all zero = defaults)
   size_t scratch_total = 0;   // bytes held by the Bufs below
+  std::vector<unsigned char> dm_host;  // what the last shift table uploaded to dm_in
   const int *dk_max = nullptr;  // [n_dm] in dm_in, of the last shift table
   Buf vis, dk, dm_in, series, pnorm, stats, counts, offsets, events, small, seglist, masks, hits, errflag, refine, calib,
       ytree;

@@ -30,3 +30,14 @@ def test_largest_shift(frbx, f0):  # noqa: F811
         with pytest.raises(frbx.FrbxError) as e:
             h.fit_segments(vis, dms, rows(max(last + 1, 0)))
         assert e.value.code == frbx.FRBX_EINVAL
+
+
+def test_no_segments_leaves_nothing_in_flight(frbx):  # noqa: F811
+    """A fit of no segments returns once the host cube is read, so the caller may release or rewrite it."""
+    import torch
+    h = frbx.Handle(np.array([1400.0, 1432.0]), 4, 16.0, 0.5)
+    vis = torch.zeros((1, 1 << 22, h.C), dtype=torch.complex64, pin_memory=True)  # 268 MB
+    st = torch.cuda.current_stream()
+    for _ in range(2):
+        assert len(h.fit_segments(vis, np.array([0.0, 50.0]), np.zeros((0, 4), np.int32))) == 0
+        assert st.query()
