@@ -40,9 +40,9 @@ FIT_DRAM_BYTES_PER_SEGMENT = None
 # covers, from an ncu capture of the vgos-profile workload; None: k_tree_mbd has changed since
 # its last capture
 TREE_MBD_DRAM_BYTES_PER_AP = None
-# the same for k_tree_mma (the tensor-core MBD pass, 2048-AP time tiles): 2.701 + 0.009 GB over
-# 4 x 20000 series-APs
-TREE_MMA_DRAM_BYTES_PER_AP = (2.700700e9 + 0.009359e9) / (4 * 20000)
+# the same for k_tree_mma (the tensor-core MBD pass, blocks of 48 columns, 2048-AP time tiles):
+# 4.232 + 0.007 GB over 4 x 20000 series-APs
+TREE_MMA_DRAM_BYTES_PER_AP = (4.232260e9 + 0.006728e9) / (4 * 20000)
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
 
 
@@ -400,7 +400,7 @@ def main():
         e1.record(stream)
         torch.cuda.synchronize()
         e2e_ms.append(e0.elapsed_time(e1))
-        d2h = 4 * len(wl.dms) + 16 + 28 * o["counts"]["events_baseline"] + \
+        d2h = 16 + 28 * o["counts"]["events_baseline"] + \
             28 * (o["counts"]["events"] - o["counts"]["events_baseline"]) + 16 * (1 + len(combos))
     e2e = max_over_ranks(statistics.mean(e2e_ms))
 
@@ -415,7 +415,7 @@ def main():
     bf16_peak = peaks["bf16_tflops_sustained"]
     if tree:
         # dominant kernel: the MBD pass of the window-tree fit (k_tree_mma on the tensor cores,
-        # or k_tree_mbd on the CUDA cores), timed per chunk with CUDA events on the library's
+        # or k_tree_mbd / k_tree16 on the CUDA cores), timed per chunk with CUDA events on the library's
         # stream it runs on; it emits every segment
         kms = statistics.mean(mbd_ms)
         achieved = flops / (kms / 1e3) / 1e12
@@ -445,7 +445,7 @@ def main():
                         "work": "2 Ls Lm per summed window + 3 Ls Lm per emitted segment"}}
         else:
             executed = n_ap * h.Ls * 5 * h.Lm * math.log2(h.Lm) + epilogue
-            roof = {"bound": "alu", "kernel": "k_tree_mbd", "achieved": achieved, "peak": own["fp32"],
+            roof = {"bound": "alu", "kernel": "k_tree16" if h.Lm == 16 else "k_tree_mbd", "achieved": achieved, "peak": own["fp32"],
                     "unit": "TFLOP/s", "frac": achieved / own["fp32"], "traffic": traffic,
                     "peak_kind": "this GPU's FP32 FMA pipe, measured by libfrbx_peaks", "work": work,
                     "executed": {"achieved": executed / (kms / 1e3) / 1e12,
