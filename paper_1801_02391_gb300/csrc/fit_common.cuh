@@ -153,14 +153,32 @@ __device__ __forceinline__ bool tile_segment(const FitArgs &a, bool list, int i,
   return true;
 }
 
-// Eq. 3 gather of one segment into X (row stride xs), weighted and rotated.
+// Eq. 3 gather of one segment into X (row stride xs), weighted and rotated.  kGatherPts points of a
+// thread side by side: with four, kGatherAps APs of each are loaded before they are added (in AP order),
+// 16 loads in flight, where one point at a time waits for every fourth AP (k_fit_fft, 20000 segments of
+// 1 to 32 APs: 2.84 -> 2.44 ms).  k_fit_direct takes one: its few registers (40) hide the loads by
+// occupancy, and its usual S-band setup has one point per thread (per-segment search of 3 baselines x
+// 101 DM trials x 4096 APs: call of 31.4 ms with one, 40.9 ms with four, which take 128 registers).
+template <int kGatherPts>
 __device__ __forceinline__ void gather_segment(const FitArgs &a, const ItemCtx &c, const Seg &s, float2 *X, int xs) {
   const int *dk = a.dk + (size_t)s.d * a.C;
   const size_t base = (size_t)s.bl * c.T + s.k0;
-  // kGatherPts points of a thread side by side, kGatherAps APs of each loaded before they are added (in
-  // AP order): 16 loads in flight, where one point at a time waited for every fourth AP (20000 segments of
-  // 1 to 32 APs: 2.84 -> 2.44 ms)
-  constexpr int kGatherPts = 4, kGatherAps = 4;
+  if constexpr (kGatherPts == 1) {
+    for (int p = threadIdx.x; p < a.C; p += blockDim.x) {
+      const float2 *src = c.vis + (base + __ldg(dk + p)) * a.C + p;
+      float2 acc = make_float2(0.f, 0.f);
+#pragma unroll 4
+      for (int i = 0; i < s.l; ++i) {
+        const float2 v = __ldg(src + (size_t)i * a.C);
+        acc.x += v.x;
+        acc.y += v.y;
+      }
+      const int n = p / a.J, j = p - n * a.J;
+      X[n * xs + j] = cmul(acc, __ldg(a.wrot + p));
+    }
+    return;
+  }
+  constexpr int kGatherAps = 4;
   for (int p0 = threadIdx.x; p0 < a.C; p0 += blockDim.x * kGatherPts) {
     const float2 *src[kGatherPts];
     float2 acc[kGatherPts];

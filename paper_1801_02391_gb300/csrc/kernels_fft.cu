@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads)
       if (threadIdx.x == 0) write_fit(a, c.out, s, -1.f, 0);
       continue;
     }
-    gather_segment(a, c, s, X, L.xs);
+    gather_segment<4>(a, c, s, X, L.xs);
     __syncthreads();
 
     // SBD transform, task (n, m1)

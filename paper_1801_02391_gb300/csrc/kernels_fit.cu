@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kFitThreads)
       if (threadIdx.x == 0) write_fit(a, c.out, s, -1.f, 0);
       continue;
     }
-    gather_segment(a, c, s, X, J);
+    gather_segment<1>(a, c, s, X, J);
     __syncthreads();
     // Eq. 5, sum over j = 1 .. J-1 for every (n, m)
     for (int o = threadIdx.x; o < N * Ls; o += blockDim.x) {
