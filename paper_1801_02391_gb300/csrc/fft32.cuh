@@ -41,28 +41,25 @@ __device__ __forceinline__ float2 csub(float2 a, float2 b) {
 
 // Radix-2 decimation-in-frequency butterflies of one stage (span S) on NP values; the
 // twiddle of butterfly K at span S is exp(-2 pi i K / (2 S)) = w32^(K * 16 / S).
-// kPacked: sums as packed pairs, which tie the registers of a value together: where a kernel is at its
-// register limit, the scalar form spills less.
-template <bool kPacked, int NP, int S, int B, int K>
+template <int NP, int S, int B, int K>
 __device__ __forceinline__ void dif_bfly(float2 (&a)[NP]) {
   const float2 u = a[B + K], v = a[B + K + S];
-  a[B + K] = kPacked ? cadd(u, v) : make_float2(u.x + v.x, u.y + v.y);
-  a[B + K + S] = twiddle32<K * (16 / S)>(kPacked ? csub(u, v) : make_float2(u.x - v.x, u.y - v.y));
-  if constexpr (K + 1 < S) dif_bfly<kPacked, NP, S, B, K + 1>(a);
+  a[B + K] = cadd(u, v);
+  a[B + K + S] = twiddle32<K * (16 / S)>(csub(u, v));
+  if constexpr (K + 1 < S) dif_bfly<NP, S, B, K + 1>(a);
 }
-template <bool kPacked, int NP, int S, int B>
+template <int NP, int S, int B>
 __device__ __forceinline__ void dif_stage(float2 (&a)[NP]) {
-  dif_bfly<kPacked, NP, S, B, 0>(a);
-  if constexpr (B + 2 * S < NP) dif_stage<kPacked, NP, S, B + 2 * S>(a);
+  dif_bfly<NP, S, B, 0>(a);
+  if constexpr (B + 2 * S < NP) dif_stage<NP, S, B + 2 * S>(a);
 }
 // In-place 32-point DFT (forward, exp(-i)); output k holds frequency bitrev5(k).
-template <bool kPacked = true>
 __device__ __forceinline__ void fft32_dif(float2 (&a)[32]) {
-  dif_stage<kPacked, 32, 16, 0>(a);
-  dif_stage<kPacked, 32, 8, 0>(a);
-  dif_stage<kPacked, 32, 4, 0>(a);
-  dif_stage<kPacked, 32, 2, 0>(a);
-  dif_stage<kPacked, 32, 1, 0>(a);
+  dif_stage<32, 16, 0>(a);
+  dif_stage<32, 8, 0>(a);
+  dif_stage<32, 4, 0>(a);
+  dif_stage<32, 2, 0>(a);
+  dif_stage<32, 1, 0>(a);
 }
 // The same 16-point DFT as fft16_dif of inputs whose upper eight are zero (left unset): the first stage
 // only copies and turns.
@@ -71,20 +68,18 @@ __device__ __forceinline__ void low_bfly(float2 (&a)[16]) {
   a[K + 8] = twiddle32<2 * K>(a[K]);
   if constexpr (K + 1 < 8) low_bfly<K + 1>(a);
 }
-template <bool kPacked = true>
 __device__ __forceinline__ void fft16_dif_low(float2 (&a)[16]) {
   low_bfly<0>(a);
-  dif_stage<kPacked, 16, 4, 0>(a);
-  dif_stage<kPacked, 16, 2, 0>(a);
-  dif_stage<kPacked, 16, 1, 0>(a);
+  dif_stage<16, 4, 0>(a);
+  dif_stage<16, 2, 0>(a);
+  dif_stage<16, 1, 0>(a);
 }
 // In-place 16-point DFT (forward, exp(-i)); output k holds frequency bitrev4(k).
-template <bool kPacked = true>
 __device__ __forceinline__ void fft16_dif(float2 (&a)[16]) {
-  dif_stage<kPacked, 16, 8, 0>(a);
-  dif_stage<kPacked, 16, 4, 0>(a);
-  dif_stage<kPacked, 16, 2, 0>(a);
-  dif_stage<kPacked, 16, 1, 0>(a);
+  dif_stage<16, 8, 0>(a);
+  dif_stage<16, 4, 0>(a);
+  dif_stage<16, 2, 0>(a);
+  dif_stage<16, 1, 0>(a);
 }
 
 static inline cudaError_t upload_w32() {

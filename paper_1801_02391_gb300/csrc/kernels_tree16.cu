@@ -16,6 +16,8 @@
 // The S-band search of 3 baselines x 101 DM trials x 4096 APs: both passes 13.0 -> 3.1 ms (the two-pass
 // form issued on few of its cycles: two serial device reads per AP, half of each CTA's threads idle).
 // Three-input maxima, a first FFT stage without its zeros and reads of two points: call 4.64 -> 4.55 ms.
+// Every sum (FFTs and windows) as packed pairs: kernel 2.98 -> 2.75 ms, call 4.40 -> 4.15 ms (the windows' sums
+// alone 2.94 ms).  Four CTAs per SM at 128 registers spill: 5.78 ms.
 #include "fit_common.cuh"
 #include "fft32.cuh"
 
@@ -50,7 +52,7 @@ __global__ void __launch_bounds__(kThreads16, 3)
   float4 *Y = reinterpret_cast<float4 *>(smem);           // [kAps][kPairs][Ls + 2] slots 2p, 2p + 1
   float2 *X = reinterpret_cast<float2 *>(Y + kAps * kYAp);  // [kAps][N][xs]
   float2 *stw = X + kAps * N * xs;                        // [kPS][xs]
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x;
   for (int i = tid; i < kAps * kYAp; i += kThreads16) Y[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int i = tid; i < kAps * N * xs; i += kThreads16) X[i] = make_float2(0.f, 0.f);
   for (int i = tid; i < kPS * a.J1 * 32; i += kThreads16) {
@@ -155,7 +157,7 @@ __global__ void __launch_bounds__(kThreads16, 3)
       g[2 * p] = cfma(make_float2(0.f, 0.f), make_float2(y.x, y.y), unit);
       g[2 * p + 1] = cfma(make_float2(0.f, 0.f), make_float2(y.z, y.w), unit);
     }
-    fft16_dif_low<false>(g);
+    fft16_dif_low(g);
   };
 
   float2 ga[16], gb[16], h2[16];  // G_1 of two consecutive APs, G_2 of the last odd AP
@@ -179,7 +181,7 @@ __global__ void __launch_bounds__(kThreads16, 3)
           A[j2 + 1] = cfma(A[j2 + 1], make_float2(x.z, x.w), make_float2(w.z, w.w));
         }
       }
-      fft32_dif<false>(A);
+      fft32_dif(A);
 #pragma unroll
       for (int i = 0; i < 32; ++i) yw[2 * kPS * bitrev5(i)] = A[i];
     }
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(kThreads16, 3)
       emit(0, k, ga);
       if (t.nlev >= 1) {
 #pragma unroll
-        for (int c = 0; c < 16; ++c) acc[c] = make_float2(gb[c].x + ga[c].x, gb[c].y + ga[c].y);
+        for (int c = 0; c < 16; ++c) acc[c] = cadd(gb[c], ga[c]);
         emit(1, k, acc);
       }
       if (more) {
@@ -209,8 +211,8 @@ __global__ void __launch_bounds__(kThreads16, 3)
       if (t.nlev >= 1) {
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
-          const float2 g = make_float2(ga[c].x + gb[c].x, ga[c].y + gb[c].y), p = h2[c];
-          acc[c] = make_float2(p.x + g.x, p.y + g.y);
+          const float2 g = cadd(ga[c], gb[c]);
+          acc[c] = cadd(h2[c], g);
           h2[c] = g;
         }
         emit(1, k + 1, h2);
@@ -223,8 +225,8 @@ __global__ void __launch_bounds__(kThreads16, 3)
     for (int e = 3; e <= E; ++e) {
 #pragma unroll
       for (int c = 0; c < 16; ++c) {
-        const float2 g = acc[c], p = deep[e - 3][c];
-        acc[c] = make_float2(p.x + g.x, p.y + g.y);
+        const float2 g = acc[c];
+        acc[c] = cadd(deep[e - 3][c], g);
         deep[e - 3][c] = g;
       }
       emit(e, i + 3, acc);
