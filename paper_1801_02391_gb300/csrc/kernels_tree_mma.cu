@@ -719,6 +719,9 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
       if (lane == 0) tc::mbar_arrive(&bar_accempty[slot]);
     }
     if (!ok) *abortp = 1;
+    // the last anchor stores are done before the tensor memory is given back: the next CTA on this SM
+    // gets the same columns
+    tm_wait_st();
     }
   }
 
