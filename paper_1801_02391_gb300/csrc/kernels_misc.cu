@@ -167,8 +167,10 @@ __global__ void __launch_bounds__(256) k_stats_count(StatsArgs a) {
   if (fast) c = series_pair(a, s, d, off).hi;
   for (int pass = 0; fast && pass < 2; ++pass) {
     Sum3 s1, s2;
+    bool differ = false;
     for (int i = threadIdx.x; i < nv; i += blockDim.x) {
       const Pair x = minus(series_pair(a, s, d, off + i), c, {0.f, 0.f});
+      differ = differ || x.hi != 0.f;
       s1.add(x.hi);
       s1.add(x.lo);
       const float q = __fmul_rn(x.hi, x.hi);
@@ -180,8 +182,9 @@ __global__ void __launch_bounds__(256) k_stats_count(StatsArgs a) {
     mean = (double)c + shift;
     const double var = fmax(t2 / nv - shift * shift, 0.0);
     sd = sqrt(var);
-    // squares within FP32 with room for their rounding terms (or all equal); false for NaN
-    fast = t2 == 0.0 || (t2 >= 1e-18 * nv && t2 <= 1e28);
+    // squares within FP32 with room for their rounding terms, or all equal (no difference at all: squares
+    // that vanish are not it); false for NaN
+    fast = __syncthreads_or(differ) == 0 || (t2 >= 1e-18 * nv && t2 <= 1e28);
     if (shift * shift <= 16.0 * var) break;  // c near the mean: nothing cancelled
     if (pass == 1) fast = fast && shift * shift <= 1e6 * var;
     c = (float)mean;
