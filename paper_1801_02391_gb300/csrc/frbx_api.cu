@@ -1961,7 +1961,10 @@ extern "C" int frbx_search_batch(frbx_batch *b, const frbx_scan *scans, int32_t 
   for (int i = 0; i < n_scans; ++i) {
     if (tree_lev[(size_t)plan[(size_t)i].setup] < 0) continue;
     const frbx::TreeArgs &tt = truns[(size_t)i].t;
+    // the launches of a scan's chunks hold where its series list starts and how long it is: the number of
+    // trials that leave an AP
     key += "|t" + std::to_string(i) + ":" + std::to_string(truns[(size_t)i].chunk) + ":" +
+           std::to_string(truns[(size_t)i].ser.size()) + ":" + std::to_string(tser_off[(size_t)i]) + ":" +
            std::to_string((uintptr_t)setups[(size_t)plan[(size_t)i].setup]->ytree.p) + ":" +
            std::to_string((uintptr_t)b->tree_ser.p) + "/";
     key.append(reinterpret_cast<const char *>(&tt), sizeof(tt));
