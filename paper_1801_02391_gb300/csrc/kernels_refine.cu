@@ -181,19 +181,21 @@ __device__ __forceinline__ void refine_walk(const RefineArgs &r, int cand, int b
     const int n = c / r.J, j = c - n * r.J;
     const RefinePoint pt = r.pt[c];
     const double u = t0 + dm * pt.ddm;
-    // integer part and fraction of u (saturates; 0 for NaN, which no tap test passes below)
-    int k0 = __double2int_rd(u);
-    double fr = u - (double)k0;
+    // integer part and fraction of u; 0 where |u| is 2^30 or more, infinite or NaN (by its exponent: no FP64
+    // operation), whose samples are taken one by one, each position tested and each phase evaluated in FP64
+    const bool near = (__double2hiint(u) & 0x7fffffff) < 0x41d00000;
+    int k0 = near ? __double2int_rd(u) : 0;
+    double fr = near ? u - (double)k0 : 0.0;
     if (fr >= 1.0) {  // u just below an integer that u + i rounds to
       ++k0;
       fr = 0.0;
     }
     const unsigned long long fr64 = unit_fraction(fr);
     // |u + i| < 2^e is rounded by 2^(e - 54) at most: 2^(e + 2) units of 2^-56, here eight times that
-    const bool small = k0 > -(1 << 20) && k0 < (1 << 20) && l < (1 << 20);
+    const bool small = near && k0 > -(1 << 20) && k0 < (1 << 20) && l < (1 << 20);
     const unsigned dw8 = small ? 32u << (32 - __clz(abs(k0) + l + 1)) : 0xffffffffu;
     float frf;
-    const bool steady = round_fraction(fr64, dw8, round_zmax(dw8), frf);
+    const bool steady = round_fraction(fr64, dw8, round_zmax(dw8), frf) && small;
     float w[4], dw[4];
     cr_weights(frf, w, dw);
     const float f0h = s_f0[n].x, f0l = s_f0[n].y;  // f0_n t_ap
@@ -204,10 +206,11 @@ __device__ __forceinline__ void refine_walk(const RefineArgs &r, int cand, int b
       bl = (float)(p - (double)bh);
     }
     // samples [lo, hi) of a steady point have their four taps in the cube
-    const int lo = max(0, 1 - k0), hi = min(l, r.T - 2 - k0);
+    const int lo = steady ? max(0, 1 - k0) : 0, hi = steady ? min(l, r.T - 2 - k0) : 0;
     if (steady && (lo > 0 || hi < l)) edge |= l > 0;
     const ChanPhase ph = s_ph[n];
-    const BlPhase bp = s_bl;
+    BlPhase bp = s_bl;
+    if (!near) bp.zmax = -1;  // no phase from k0
     // offset + j step + rate (k0 + fr), modulo one cycle; the rate is signed
     unsigned long long cyc = ph.offset + (unsigned long long)j * bp.step + (unsigned long long)(long long)k0 * ph.rate +
                              (unsigned long long)ph.whole * fr64 + __umul64hi(ph.rate, fr64) -
