@@ -222,12 +222,13 @@ __device__ __forceinline__ void refine_walk(const RefineArgs &r, int cand, int b
       float red, fx = 0.f;
       bool sure = round_fraction(ph_i, bp.slack8, bp.zmax, red);
       if (kAdjoint) {
-        // f0_n t_ap (u + i) = (bh + bl) + i (f0h + f0l), to about 2^-44 of itself
+        // f0_n t_ap (u + i) = (bh + bl) + i (f0h + f0l), to about 2^-46 of the two terms (which cancel in windows
+        // that start before the cube); i is a float up to 2^24
         float se;
         const float fi = (float)i, p = __fmul_rn(fi, f0h), pe = fmaf(fi, f0h, -p);
-        const float sh = two_sum(bh, p, se), sl = se + (bl + fmaf(fi, f0l, pe)), d = fabsf(sh) * 0x1p-42f;
+        const float sh = two_sum(bh, p, se), sl = se + (bl + fmaf(fi, f0l, pe)), d = (fabsf(bh) + p) * 0x1p-42f;
         fx = sh + (sl - d);
-        sure = sure && fx == sh + (sl + d);
+        sure = sure && i <= (1 << 24) && fx == sh + (sl + d);
       }
       if (!sure) {
         // the FP64 expressions, their operations spelled out (one branch for both: the shorter alone
