@@ -22,7 +22,6 @@ namespace frbx {
 
 constexpr int kFftThreads = 128;      // four CTAs per SM
 constexpr int kFftWideThreads = 512;  // one CTA per SM: a list shorter than the GPU
-constexpr int kFftWarps = kFftWideThreads / 32;
 constexpr int kFftWideRows = 2;       // longest list of the wide form, in segments per SM
 
 struct FftSmem {
@@ -30,7 +29,7 @@ struct FftSmem {
   size_t bytes;
 };
 
-__host__ __device__ inline FftSmem fft_smem_layout(int N, int Ls, int Lm, int J1) {
+__host__ __device__ inline FftSmem fft_smem_layout(int N, int Ls, int Lm, int J1, int threads) {
   FftSmem l;
   const int JP = J1 * 32;
   l.xs = JP + 1;   // odd stride: column reads of 8 channel rows hit distinct banks
@@ -38,7 +37,7 @@ __host__ __device__ inline FftSmem fft_smem_layout(int N, int Ls, int Lm, int J1
   l.ts = JP + 1;
   l.bytes = sizeof(float2) * ((size_t)N * l.xs + (size_t)N * l.ys + (size_t)(Ls / 32) * l.ts +
                               (size_t)N * (Lm / 32)) +
-            2 * kFftWarps * sizeof(int);  // block reduction
+            2 * (threads < 256 ? 8 : threads / 32) * sizeof(int);  // block reduction (at least 64 bytes)
   return l;
 }
 
@@ -51,13 +50,13 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads)
   const int PS = Ls >> 5, PM = Lm >> 5;
   const int lps = __ffs(PS) - 1, lpm = __ffs(PM) - 1;
   const int JP = a.J1 * 32;
-  const FftSmem L = fft_smem_layout(N, Ls, Lm, a.J1);
+  const FftSmem L = fft_smem_layout(N, Ls, Lm, a.J1, kThreads);
   float2 *X = reinterpret_cast<float2 *>(smem);  // [N][xs]
   float2 *Y = X + N * L.xs;                      // [N][ys]
   float2 *stw = Y + N * L.ys;                    // [PS][ts]
   float2 *mtw = stw + PS * L.ts;                 // [N][PM]
   float *rp = reinterpret_cast<float *>(mtw + N * PM);
-  int *ri = reinterpret_cast<int *>(rp + kFftWarps);
+  int *ri = reinterpret_cast<int *>(rp + kThreads / 32);
 
   for (int i = threadIdx.x; i < N * L.xs; i += blockDim.x) X[i] = make_float2(0.f, 0.f);
   for (int i = threadIdx.x; i < PS * JP; i += blockDim.x) {
@@ -174,7 +173,7 @@ static cudaError_t launch_one(const FitArgs &a, dim3 grid, size_t smem, int list
 
 cudaError_t launch_fit_fft(const FitArgs &a, int n_bl, bool list_mode, cudaStream_t st, int64_t *launches) {
   if (!fft_supported(a.Ls, a.Lm, a.J) || a.occ > 4 || a.occ < 1) return cudaErrorInvalidConfiguration;
-  const size_t smem = fft_smem_layout(a.N, a.Ls, a.Lm, a.J1).bytes;
+  size_t smem = fft_smem_layout(a.N, a.Ls, a.Lm, a.J1, kFftThreads).bytes;
   if (smem > max_smem_optin()) return cudaErrorInvalidConfiguration;
   dim3 grid;
   if (!fit_grid(a, n_bl, list_mode, &grid)) return cudaErrorInvalidConfiguration;
@@ -182,8 +181,12 @@ cudaError_t launch_fit_fft(const FitArgs &a, int n_bl, bool list_mode, cudaStrea
   const bool full = a.m_lo == 0 && a.m_len == a.Ls && a.q_lo == 0 && a.q_len == a.Lm;
   const int list = list_mode ? 1 : 0;
   cudaError_t e;
-  // one segment per CTA and no more than kFftWideRows per SM: the wide form
-  const bool wide = list_mode && a.tile == 1 && a.n_seg <= (long long)kFftWideRows * sm_count();
+  // one segment per CTA and no more than kFftWideRows per SM: the wide form, where its reduction over 16
+  // warps (64 bytes more) fits too, with 1 KB left for the kernel's own tables
+  const size_t wide_smem = fft_smem_layout(a.N, a.Ls, a.Lm, a.J1, kFftWideThreads).bytes;
+  const bool wide = list_mode && a.tile == 1 && a.n_seg <= (long long)kFftWideRows * sm_count() &&
+                    wide_smem + 1024 <= max_smem_optin();
+  if (wide) smem = wide_smem;
   if (wide && a.occ == 1) e = full ? launch_one<1, true, false, kFftWideThreads>(a, grid, smem, list, st) : launch_one<1, false, false, kFftWideThreads>(a, grid, smem, list, st);
   else if (wide && a.occ == 2) e = full ? launch_one<2, true, false, kFftWideThreads>(a, grid, smem, list, st) : launch_one<2, false, false, kFftWideThreads>(a, grid, smem, list, st);
   else if (wide) e = full ? launch_one<4, true, false, kFftWideThreads>(a, grid, smem, list, st) : launch_one<4, false, false, kFftWideThreads>(a, grid, smem, list, st);
@@ -197,7 +200,7 @@ cudaError_t launch_fit_fft(const FitArgs &a, int n_bl, bool list_mode, cudaStrea
 cudaError_t launch_fit_fft_batch(const FitArgs &a, const BatchScan *scans, int n_scans, long long total,
                                  unsigned int *counter, int ctas_per_sm, cudaStream_t st, int64_t *launches) {
   if (!fft_supported(a.Ls, a.Lm, a.J) || a.occ > 4 || a.occ < 1) return cudaErrorInvalidConfiguration;
-  const size_t smem = fft_smem_layout(a.N, a.Ls, a.Lm, a.J1).bytes;
+  const size_t smem = fft_smem_layout(a.N, a.Ls, a.Lm, a.J1, kFftThreads).bytes;
   if (smem > max_smem_optin()) return cudaErrorInvalidConfiguration;
   if (total <= 0) return cudaSuccess;
   const int per_sm = ctas_per_sm > 0 ? ctas_per_sm : 4;
