@@ -86,15 +86,10 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
   return t;
 }
 
-// Exact sum of two floats: a + b = s + e (Knuth's two-sum), and the same for |a| >= |b|
+// Exact sum of two floats: a + b = s + e (Knuth's two-sum)
 __device__ __forceinline__ float two_sum(float a, float b, float &e) {
   const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
-  return s;
-}
-__device__ __forceinline__ float fast_two_sum(float a, float b, float &e) {
-  const float s = __fadd_rn(a, b);
-  e = __fsub_rn(b, __fsub_rn(s, a));
   return s;
 }
 // a float pair hi + lo (|lo| at most half a unit in the last place of hi: about 48 bits)
@@ -117,27 +112,44 @@ struct Sum3 {
   __device__ __forceinline__ double value() const { return (double)s + ((double)e + (double)f); }
 };
 
-// series_value as a pair
-__device__ __forceinline__ Pair series_pair(const StatsArgs &a, int s, int d, int slot) {
-  if (!a.masks) return {a.series[((size_t)s * a.n_dm + d) * a.S_tot + slot].amp, 0.f};
-  const unsigned long long mask = a.masks[s];
-  Pair v = {0.f, 0.f};
-  for (int b = 0; b < a.n_bl; ++b)
-    if ((mask >> b) & 1ull) {
-      float e;
-      v.hi = two_sum(v.hi, a.series[((size_t)b * a.n_dm + d) * a.S_tot + slot].amp, e);
-      v.lo += e;
-    }
-  v.hi = fast_two_sum(v.hi, v.lo, v.lo);
+// series_value as three floats (their sum to about 2^-70 of the amplitudes; a baseline's is one)
+struct Tri {
+  float hi = 0.f, mid = 0.f, lo = 0.f;
+};
+template <bool kCombo>
+__device__ __forceinline__ Tri series_tri(const StatsArgs &a, int s, int d, int slot) {
+  Tri v;
+  if constexpr (!kCombo) {
+    v.hi = a.series[((size_t)s * a.n_dm + d) * a.S_tot + slot].amp;
+  } else {
+    const unsigned long long mask = a.masks[s];
+    for (int b = 0; b < a.n_bl; ++b)
+      if ((mask >> b) & 1ull) {
+        float e, g;
+        v.hi = two_sum(v.hi, a.series[((size_t)b * a.n_dm + d) * a.S_tot + slot].amp, e);
+        v.mid = two_sum(v.mid, e, g);
+        v.lo += g;
+      }
+  }
   return v;
 }
 
-// v - c - (m.hi + m.lo)
-__device__ __forceinline__ Pair minus(Pair v, float c, Pair m) {
-  float e1, e2;
-  const float s1 = two_sum(v.hi, -c, e1), s2 = two_sum(s1, -m.hi, e2);
+// v - c - (m.hi + m.lo) to about 2^-46 of itself, of m and of 2^-24 v (v.mid may be as large as the result)
+template <bool kCombo>
+__device__ __forceinline__ Pair minus(Tri v, float c, Pair m) {
+  float e1, e2, rest;
+  const float s1 = two_sum(v.hi, -c, e1);
+  float s2 = two_sum(s1, -m.hi, e2);
+  if constexpr (kCombo) {
+    float f1, f2;
+    const float t = two_sum(e1, v.mid, f1);
+    s2 = two_sum(s2, t, f2);
+    rest = (e2 + f2) + ((f1 + v.lo) - m.lo);
+  } else {
+    rest = e2 + (e1 - m.lo);
+  }
   Pair r;
-  r.hi = fast_two_sum(s2, e2 + (e1 + (v.lo - m.lo)), r.lo);
+  r.hi = two_sum(s2, rest, r.lo);
   return r;
 }
 
@@ -148,12 +160,17 @@ __host__ __device__ __forceinline__ size_t hit_words(int S_tot, int n_win) { ret
 // crossings P = (A - mean) / std > threshold, their count and one bit each; optionally writes P.
 //
 // FP64 runs at a 64th of FP32's rate here, and a division of it per slot was most of this kernel and of
-// the one that writes the events.  The sums are taken of the differences from the first amplitude (and of
-// their squares, with the products' rounding) in three floats each, P is formed in float pairs, and
-// both are as exact as the FP64 they replace; P's pair decides a crossing unless it is within 1e-9 of
-// the threshold, which the FP64 expression then decides.  Series whose squares FP32 cannot hold, or with a
+// the one that writes the events.  The results are those of FP64 all the same:
+//  * mean and std come from the differences from c, an estimate of the mean, and their squares, without
+//    rounding errors above 2^-48 of a term and summed in three floats each; c is taken anew where it is
+//    farther than one std from the mean, so the shift of the squares loses one bit at most;
+//  * P is formed in float pairs, and taken when every value within their error rounds to the same float;
+//    otherwise the FP64 expression is evaluated (about one slot in 10^5);
+//  * a crossing within 1e-9 of the threshold is decided by the FP64 expression.
+// Series whose squares FP32 cannot hold, that vary by less than a float resolves, or with a
 // value that is not finite, take FP64 throughout.  With k_events and k_scan below, for 2.1 million slots
 // of baselines and four combinations: 0.71 -> 0.45 ms.
+template <bool kCombo>
 __global__ void __launch_bounds__(256) k_stats_count(StatsArgs a) {
   __shared__ double red[32];
   const int w = blockIdx.x, d = blockIdx.y, s = blockIdx.z;
@@ -161,32 +178,41 @@ __global__ void __launch_bounds__(256) k_stats_count(StatsArgs a) {
   const int off = a.win_off[w];
   const size_t sid = ((size_t)s * a.n_dm + d) * a.n_win + w;
   unsigned *const bits = a.hits + ((size_t)s * a.n_dm + d) * hit_words(a.S_tot, a.n_win) + (off >> 5) + w;
-  double mean = 0.0, sd = 0.0, shift = 0.0;  // shift: mean - c
+  double mean = 0.0, sd = 0.0;
   float c = 0.f;
   bool fast = nv > 0;
-  if (fast) c = series_pair(a, s, d, off).hi;
+  if (fast) {  // the mean of 32 slots spread over the series (every warp the same)
+    c = series_tri<kCombo>(a, s, d, off + (int)((long long)(threadIdx.x & 31) * nv >> 5)).hi;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    c *= 0.03125f;
+  }
   for (int pass = 0; fast && pass < 2; ++pass) {
     Sum3 s1, s2;
     bool differ = false;
     for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-      const Pair x = minus(series_pair(a, s, d, off + i), c, {0.f, 0.f});
+      const Pair x = minus<kCombo>(series_tri<kCombo>(a, s, d, off + i), c, {0.f, 0.f});
       differ = differ || x.hi != 0.f;
-      s1.add(x.hi);
-      s1.add(x.lo);
       const float q = __fmul_rn(x.hi, x.hi);
+      s1.add(x.hi);
       s2.add(q);
-      s2.add(fmaf(2.f * x.hi, x.lo, fmaf(x.hi, x.hi, -q)));
+      s2.add(fmaf(x.hi, x.hi, -q));
+      if (x.lo != 0.f) {
+        const float p = __fmul_rn(2.f * x.hi, x.lo);
+        s1.add(x.lo);
+        s2.add(p);
+        s2.add(fmaf(x.lo, x.lo, fmaf(2.f * x.hi, x.lo, -p)));
+      }
     }
     const double t1 = block_sum(s1.value(), red), t2 = block_sum(s2.value(), red);
-    shift = t1 / nv;
+    const double shift = t1 / nv, var = fmax(t2 / nv - shift * shift, 0.0);
     mean = (double)c + shift;
-    const double var = fmax(t2 / nv - shift * shift, 0.0);
     sd = sqrt(var);
     // squares within FP32 with room for their rounding terms, or all equal (no difference at all: squares
     // that vanish are not it); false for NaN
     fast = __syncthreads_or(differ) == 0 || (t2 >= 1e-18 * nv && t2 <= 1e28);
-    if (shift * shift <= 16.0 * var) break;  // c near the mean: nothing cancelled
-    if (pass == 1) fast = fast && shift * shift <= 1e6 * var;
+    if (shift * shift <= var) break;
+    if (pass == 1) fast = false;
     c = (float)mean;
   }
   if (!fast && nv > 0) {
@@ -202,6 +228,8 @@ __global__ void __launch_bounds__(256) k_stats_count(StatsArgs a) {
   }
   const double inv = sd > 0.0 ? 1.0 / sd : 0.0;
   const Pair m = to_pair(mean - (double)c), r = to_pair(inv), th = to_pair(a.threshold);
+  // P's error is below 2^-44 of itself and of m / sd; 1e-37: products that FP32 holds with fewer bits
+  const float err0 = fmaf(fabsf(m.hi) * r.hi, 0x1p-43f, 1e-37f);
   int cnt = 0;
   for (int i0 = threadIdx.x & ~31; i0 < nv; i0 += blockDim.x) {  // 32 slots of a warp: one word
     const int i = i0 + (threadIdx.x & 31);
@@ -210,12 +238,18 @@ __global__ void __launch_bounds__(256) k_stats_count(StatsArgs a) {
     if (i < nv) {
       bool sure = fast && sd > 0.0;
       if (sure) {
-        const Pair x = minus(series_pair(a, s, d, off + i), c, m);
+        const Tri v = series_tri<kCombo>(a, s, d, off + i);
+        const Pair x = minus<kCombo>(v, c, m);
         const float ph = __fmul_rn(x.hi, r.hi), pl = fmaf(x.hi, r.lo, fmaf(x.lo, r.hi, fmaf(x.hi, r.hi, -ph)));
-        pn = ph + pl;
         const float g = (ph - th.hi) + (pl - th.lo);
         hit = g > 0.f;
-        sure = fabsf(g) > 1e-9f * (1.f + fabsf(ph));  // false for NaN
+        // (the FP64 sum of a combination is rounded itself: 2^-53 of each amplitude); false for NaN
+        sure = fabsf(g) > 1e-9f * (1.f + fabsf(ph)) + (kCombo ? 1e-14f * fabsf(v.hi) * r.hi : 0.f);
+        if (a.pnorm) {
+          const float err = fmaf(fabsf(ph), 0x1p-43f, err0);
+          pn = ph + (pl - err);
+          sure = sure && pn == ph + (pl + err);
+        }
       }
       if (!sure) {
         const double p = sd > 0.0 ? (series_value(a, s, d, off + i) - mean) / sd : 0.0;
@@ -328,7 +362,9 @@ size_t stats_hit_bytes(int n_series, int n_dm, int S_tot, int n_win) {
 
 cudaError_t launch_stats_count(const StatsArgs &a, cudaStream_t st, int64_t *launches) {
   if (a.n_series == 0 || a.n_dm == 0 || a.n_win == 0) return cudaSuccess;
-  k_stats_count<<<dim3(a.n_win, a.n_dm, a.n_series), 256, 0, st>>>(a);
+  const dim3 grid(a.n_win, a.n_dm, a.n_series);
+  if (a.masks) k_stats_count<true><<<grid, 256, 0, st>>>(a);
+  else k_stats_count<false><<<grid, 256, 0, st>>>(a);
   ++*launches;
   return cudaGetLastError();
 }

@@ -1,6 +1,6 @@
 """Normalised power and crossings where the float-pair arithmetic of the normalisation is at its limits: series
-whose amplitudes differ by so little that FP32 squares of the differences vanish, and amplitudes that are not
-finite.  P is recomputed in FP64 from the amplitudes the search returns."""
+whose amplitudes differ by so little that FP32 squares of the differences vanish, or by little more than a float
+resolves, the rounding of P, and amplitudes that are not finite.  P is recomputed in FP64 from the amplitudes the search returns."""
 import numpy as np
 import pytest
 
@@ -34,6 +34,33 @@ def test_differences_that_cancel(frbx):  # noqa: F811
     assert ((amp[:, 1] - amp[:, 0]) ** 2 == 0).all() and (amp[:, 0] != amp[:, 1]).sum() > 16
     _check(out, combos, off)
     assert (np.abs(out["pnorm"][:, 0]) == (amp[:, :1] != amp[:, 1:])).all()
+
+
+def test_p_is_the_fp64_expression_rounded(frbx):  # noqa: F811
+    """Every slot made a crossing: the events hold (A - mean) / std in FP64, rounded, and so does P.  The first slots
+    lie several std above the mean."""
+    import torch
+    n_bl, T = 48, 8192
+    wl = synth.make_small(T=T, n_bl=n_bl, dms=np.arange(10.0))
+    gen = torch.Generator("cuda").manual_seed(5)
+    vis = torch.view_as_complex(torch.randn((n_bl, T, wl.C, 2), device="cuda", generator=gen))
+    vis[:, :60] *= 1.3
+    out = frbx.Handle.from_workload(wl).search(vis, wl.dms, [1], threshold=-100.0, nwin_min=2, want_series=True,
+                                               want_events=True)
+    ev = out["events"]
+    assert len(ev) == (out["series"]["amp"] >= 0).sum() > 3_900_000
+    assert np.array_equal(ev["pnorm"], out["pnorm"][ev["series"], ev["dm_idx"], ev["k0"]])
+
+
+@pytest.mark.parametrize("part", [1e-4, 1e-6, 2e-7])
+def test_nearly_constant_series(frbx, part):  # noqa: F811
+    """Amplitudes that vary by little more than a float resolves, alone and in combinations."""
+    def edit(vis):
+        rng = np.random.default_rng(6)
+        vis[:] = vis[:, :1] * (1.0 + part * rng.standard_normal((vis.shape[0], vis.shape[1], 1))).astype(np.float32)
+    out, combos, off = _run(frbx, 300, edit)
+    _check(out, combos, off)
+    assert out["counts"]["events"] > 0
 
 
 @pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
