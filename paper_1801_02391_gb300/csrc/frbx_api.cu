@@ -48,11 +48,17 @@ cudaError_t ensure(frbx_handle::Buf &b, size_t bytes) {
 }
 
 // The same for a handle's own scratch, counted against its scratch cap (frbx_limits): growing
-// past the cap fails as an allocation failure (FRBX_ENOMEM) and keeps the old buffer.
+// past the cap fails as an allocation failure (FRBX_ENOMEM) and keeps the old buffer.  The hit mask
+// of the normalisation is given up first: what it saves is time only.
 cudaError_t ensure(frbx_handle *h, frbx_handle::Buf &b, size_t bytes) {
   if (b.bytes >= bytes && b.p) return cudaSuccess;
   const size_t want = std::max<size_t>(bytes, 256);
   const size_t cap = (size_t)h->lim.scratch_cap_bytes;
+  if (cap > 0 && h->scratch_total - b.bytes + want > cap && &b != &h->hits && h->hits.p) {
+    h->scratch_total -= h->hits.bytes;
+    cudaFree(h->hits.p);
+    h->hits = {};
+  }
   if (cap > 0 && h->scratch_total - b.bytes + want > cap) return cudaErrorMemoryAllocation;
   h->scratch_total -= b.bytes;
   const cudaError_t e = ensure(b, want);
@@ -491,7 +497,7 @@ void frbx_destroy(frbx_handle *h) {
   for (cudaEvent_t e : h->vis_ev)
     if (e) cudaEventDestroy(e);
   if (h->copy_st) cudaStreamDestroy(h->copy_st);
-  frbx_handle::Buf *bufs[] = {&h->vis, &h->dk, &h->dm_in, &h->series, &h->pnorm, &h->stats,
+  frbx_handle::Buf *bufs[] = {&h->vis, &h->dk, &h->series, &h->pnorm, &h->stats,
                               &h->counts, &h->offsets, &h->events, &h->small, &h->seglist, &h->masks, &h->hits,
                               &h->errflag, &h->refine, &h->calib, &h->ytree};
   for (auto *b : bufs)
@@ -554,13 +560,17 @@ namespace {
 // step of Eq. 1-2 is monotonic in the frequency, so the largest shift is that of the lowest point: the
 // host evaluates it with the kernel's operations and sends it along with the trials, where reducing the
 // table on the device cost a launch, a copy back and a stop of the stream (a call with 40 segments: 92 -> 69 us).
+// h->small holds the trials, then their largest shifts; a search of n_win windows later puts its window
+// tables over the trials, which only the table's kernel reads.
 int run_shift_table(frbx_handle *h, const double *dm, int n_dm, std::vector<int> *dk_max,
-                    cudaStream_t st) {
+                    cudaStream_t st, int n_win = 0) {
   for (int d = 0; d < n_dm; ++d)
     if (!(dm[d] >= 0) || !std::isfinite(dm[d])) return fail(h, FRBX_EINVAL, "DM trials must be finite and >= 0");
-  // trials, then their largest shifts, in one copy
+  // one copy: trials, then their largest shifts
   const size_t b_dm = sizeof(double) * (size_t)n_dm, b_in = b_dm + sizeof(int) * (size_t)n_dm;
-  FRBX_CK(h, ensure(h, h->dm_in, b_in));
+  const size_t b_tab = sizeof(int) * (3 * frbx::kMaxWin + (size_t)n_dm * n_win);
+  const size_t o_max = std::max(b_dm, (b_tab + 7) & ~(size_t)7);
+  FRBX_CK(h, ensure(h, h->small, o_max + b_in - b_dm));
   FRBX_CK(h, ensure(h, h->dk, sizeof(int) * (size_t)n_dm * h->C));
   const double inv_fref2 = 1.0 / (h->f_ref * h->f_ref), f_low = *std::min_element(h->f.begin(), h->f.end());
   dk_max->resize((size_t)n_dm);
@@ -570,9 +580,10 @@ int run_shift_table(frbx_handle *h, const double *dm, int n_dm, std::vector<int>
   in.resize(b_in);
   std::memcpy(in.data(), dm, b_dm);
   std::memcpy(in.data() + b_dm, dk_max->data(), b_in - b_dm);
-  FRBX_CK(h, cudaMemcpyAsync(h->dm_in.p, in.data(), b_in, cudaMemcpyHostToDevice, st));
-  h->dk_max = (const int *)((const unsigned char *)h->dm_in.p + b_dm);
-  FRBX_CK(h, frbx::launch_shift_table(h->d_f, h->C, h->f_ref, (const double *)h->dm_in.p, n_dm, h->t_ap,
+  unsigned char *d_in = (unsigned char *)h->small.p + o_max - b_dm;
+  FRBX_CK(h, cudaMemcpyAsync(d_in, in.data(), b_in, cudaMemcpyHostToDevice, st));
+  h->dk_max = (const int *)(d_in + b_dm);
+  FRBX_CK(h, frbx::launch_shift_table(h->d_f, h->C, h->f_ref, (const double *)d_in, n_dm, h->t_ap,
                                       (int *)h->dk.p, nullptr, st, &h->launches));
   return FRBX_OK;
 }
@@ -728,8 +739,10 @@ int run_stats(frbx_handle *h, StatsArgs sa, cudaStream_t st, std::vector<frbx_ev
   FRBX_CK(h, ensure(h, h->stats, sizeof(double) * 2 * ns));
   FRBX_CK(h, ensure(h, h->counts, sizeof(int) * (ns + 1)));
   FRBX_CK(h, ensure(h, h->offsets, sizeof(long long) * (ns + 1)));
-  FRBX_CK(h, ensure(h, h->hits, frbx::stats_hit_bytes(sa.n_series, sa.n_dm, sa.S_tot, sa.n_win)));
-  sa.hits = (unsigned *)h->hits.p;
+  // without room for the hit mask k_events finds the crossings itself
+  const bool mask = ensure(h, h->hits, frbx::stats_hit_bytes(sa.n_series, sa.n_dm, sa.S_tot, sa.n_win)) == cudaSuccess;
+  if (!mask) cudaGetLastError();
+  sa.hits = mask ? (unsigned *)h->hits.p : nullptr;
   sa.mean_std = (double *)h->stats.p;
   sa.counts = (int *)h->counts.p;
   sa.offsets = (long long *)h->offsets.p;
@@ -741,6 +754,7 @@ int run_stats(frbx_handle *h, StatsArgs sa, cudaStream_t st, std::vector<frbx_ev
   ev->resize((size_t)total);
   if (total == 0) return FRBX_OK;
   FRBX_CK(h, ensure(h, h->events, sizeof(frbx_event) * (size_t)total));
+  if (!h->hits.p) sa.hits = nullptr;  // given up for the events
   sa.events = (frbx_event *)h->events.p;
   FRBX_CK(h, frbx::launch_events(sa, st, &h->launches));
   FRBX_CK(h, cudaMemcpyAsync(ev->data(), sa.events, sizeof(frbx_event) * (size_t)total,
@@ -1245,7 +1259,7 @@ static int search_impl(frbx_handle *h, const void *vis, int32_t vis_on_device, i
   if (rc) return rc;
   std::vector<int> dkm;
   FRBX_CK(h, cudaEventRecord(h->ev[0], st));
-  rc = run_shift_table(h, dm, n_dm, &dkm, st);
+  rc = run_shift_table(h, dm, n_dm, &dkm, st, n_win);
   if (rc) return rc;
   FRBX_CK(h, cudaEventRecord(h->ev[1], st));
 
@@ -1263,7 +1277,7 @@ static int search_impl(frbx_handle *h, const void *vis, int32_t vis_on_device, i
   L.n_valid.resize((size_t)n_dm * n_win);
   for (int d = 0; d < n_dm; ++d)
     for (int w = 0; w < n_win; ++w) L.n_valid[(size_t)d * n_win + w] = n_valid(T, windows[w], dkm[(size_t)d]);
-  // small tables: win_len | win_off | win_step | n_valid | masks
+  // small tables: win_len | win_off | win_step | n_valid
   std::vector<int> tab;
   tab.insert(tab.end(), L.win_len.begin(), L.win_len.end());
   tab.resize(frbx::kMaxWin, 0);
@@ -1272,8 +1286,7 @@ static int search_impl(frbx_handle *h, const void *vis, int32_t vis_on_device, i
   tab.insert(tab.end(), L.win_step.begin(), L.win_step.end());
   tab.resize(3 * frbx::kMaxWin, 0);
   tab.insert(tab.end(), L.n_valid.begin(), L.n_valid.end());
-  FRBX_CK(h, ensure(h, h->small, sizeof(int) * tab.size() + 4096));
-  int *d_tab = (int *)h->small.p;
+  int *d_tab = (int *)h->small.p;  // run_shift_table left room for it
   FRBX_CK(h, cudaMemcpyAsync(d_tab, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, st));
   const size_t n_series_el = (size_t)n_bl * n_dm * L.S_tot;
   FRBX_CK(h, ensure(h, h->series, sizeof(frbx_seg) * n_series_el));
@@ -1675,7 +1688,7 @@ extern "C" int frbx_search_batch(frbx_batch *b, const frbx_scan *scans, int32_t 
     frbx_handle *h = setups[g];
     h->err.clear();
     int rc = check_params(h, &p, 64, &fa[g]);
-    if (!rc) rc = run_shift_table(h, dm, n_dm, &dkm[g], st);
+    if (!rc) rc = run_shift_table(h, dm, n_dm, &dkm[g], st, n_win);
     if (rc) return bfail(b, rc, "setup " + std::to_string(g) + ": " + h->err);
   }
   // window-tree fit where it applies (kernel 0) or is asked for (kernel 4)
@@ -2066,8 +2079,7 @@ extern "C" int frbx_search_batch(frbx_batch *b, const frbx_scan *scans, int32_t 
     h->launches = 0;
     h->tree_chunks = 0;
     int rc = FRBX_OK;
-    if (ensure(h, h->small, sizeof(int) * t2.size() + 4096) != cudaSuccess ||
-        cudaMemcpyAsync(h->small.p, t2.data(), sizeof(int) * t2.size(), cudaMemcpyHostToDevice, st) != cudaSuccess) {
+    if (cudaMemcpyAsync(h->small.p, t2.data(), sizeof(int) * t2.size(), cudaMemcpyHostToDevice, st) != cudaSuccess) {
       cudaGetLastError();
       return bfail(b, FRBX_ECUDA, "scan " + std::to_string(i) + ": table upload failed");
     }

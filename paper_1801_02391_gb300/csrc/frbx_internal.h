@@ -241,7 +241,7 @@ struct StatsArgs {
   double threshold;
   double *mean_std;        // [n_series][n_dm][n_win][2]
   int *counts;             // [n_series * n_dm * n_win + 1]
-  unsigned *hits;          // one bit per valid slot (stats_hit_bytes)
+  unsigned *hits;          // one bit per valid slot (stats_hit_bytes), or null
   long long *offsets;      // [n_series * n_dm * n_win + 1]
   frbx_event *events;      // output
   float *pnorm;            // optional [n_series][n_dm][S_tot]
@@ -316,8 +316,8 @@ struct frbx_handle {
   };
   frbx_limits lim{};          // frbx_set_limits (all zero = defaults)
   size_t scratch_total = 0;   // bytes held by the Bufs below
-  std::vector<unsigned char> dm_host;  // what the last shift table uploaded to dm_in
-  const int *dk_max = nullptr;  // [n_dm] in dm_in, of the last shift table
-  Buf vis, dk, dm_in, series, pnorm, stats, counts, offsets, events, small, seglist, masks, hits, errflag, refine, calib,
+  std::vector<unsigned char> dm_host;  // what the last shift table uploaded to small
+  const int *dk_max = nullptr;  // [n_dm] in small, of the last shift table
+  Buf vis, dk, series, pnorm, stats, counts, offsets, events, small, seglist, masks, hits, errflag, refine, calib,
       ytree;
 };

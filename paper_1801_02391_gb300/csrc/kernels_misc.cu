@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(256) k_stats_count(StatsArgs a) {
     }
     const unsigned bal = __ballot_sync(0xffffffffu, hit);
     if ((threadIdx.x & 31) == 0) {
-      bits[i0 >> 5] = bal;
+      if (a.hits) bits[i0 >> 5] = bal;
       cnt += __popc(bal);
     }
   }
@@ -316,7 +316,8 @@ __global__ void __launch_bounds__(1024) k_scan(const int *__restrict__ counts, l
   }
 }
 
-// The crossings of one (window, DM, series) in ascending k0, from the bits k_stats_count left.
+// The crossings of one (window, DM, series) in ascending k0, from the bits k_stats_count left or, where there
+// was no room for them, from the FP64 expression that they agree with.
 __global__ void __launch_bounds__(256) k_events(StatsArgs a) {
   __shared__ long long part[33];
   const int w = blockIdx.x, d = blockIdx.y, s = blockIdx.z;
@@ -327,12 +328,19 @@ __global__ void __launch_bounds__(256) k_events(StatsArgs a) {
   const unsigned *const bits = a.hits + ((size_t)s * a.n_dm + d) * hit_words(a.S_tot, a.n_win) + (off >> 5) + w;
   const double mean = a.mean_std[2 * sid], sd = a.mean_std[2 * sid + 1];
   long long out = a.offsets[sid];
+  const long long end = a.offsets[sid + 1];
   for (int c0 = 0; c0 < nw; c0 += blockDim.x) {
     const int q = c0 + threadIdx.x;
-    unsigned word = q < nw ? bits[q] : 0u;
+    unsigned word = 0u;
+    if (a.hits) {
+      if (q < nw) word = bits[q];
+    } else {
+      for (int i = q * 32; i < min(nv, q * 32 + 32); ++i)
+        if ((sd > 0.0 ? (series_value(a, s, d, off + i) - mean) / sd : 0.0) > a.threshold) word |= 1u << (i & 31);
+    }
     long long total;
     long long pos = out + block_exclusive(__popc(word), part, total);
-    for (; word != 0u; word &= word - 1u, ++pos) {
+    for (; word != 0u && pos < end; word &= word - 1u, ++pos) {
       const int i = q * 32 + __ffs((int)word) - 1;
       const double v = series_value(a, s, d, off + i);
       frbx_event e;
