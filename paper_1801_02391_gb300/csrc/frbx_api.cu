@@ -1507,10 +1507,9 @@ extern "C" int frbx_refine_adjoint(frbx_handle *h, const void *vis_dev, int32_t 
   return FRBX_OK;
 }
 
-extern "C" int frbx_calibrate(frbx_handle *h, const void *vis, int32_t vis_on_device, int32_t n_bl, int32_t T,
-                              int32_t k0, int32_t l, double *sbd_ns, double *mbd_ns, double *delay_ns,
-                              double *phase_rad, void *cuda_stream) {
-  if (!h) return FRBX_EINVAL;
+static int calibrate_impl(frbx_handle *h, const void *vis, int32_t vis_on_device, int32_t n_bl, int32_t T, int32_t k0,
+                          int32_t l, double *sbd_ns, double *mbd_ns, double *delay_ns, double *phase_rad,
+                          void *cuda_stream) {
   h->launches = 0;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (!sbd_ns || !mbd_ns || !delay_ns || !phase_rad) return fail(h, FRBX_EINVAL, "missing output");
@@ -1565,6 +1564,15 @@ extern "C" int frbx_calibrate(frbx_handle *h, const void *vis, int32_t vis_on_de
   std::copy(o + 2 * n_bl, o + (size_t)n_bl * (2 + N), delay_ns);
   std::copy(o + (size_t)n_bl * (2 + N), o + n_out, phase_rad);
   return FRBX_OK;
+}
+
+extern "C" int frbx_calibrate(frbx_handle *h, const void *vis, int32_t vis_on_device, int32_t n_bl, int32_t T,
+                              int32_t k0, int32_t l, double *sbd_ns, double *mbd_ns, double *delay_ns,
+                              double *phase_rad, void *cuda_stream) {
+  if (!h) return FRBX_EINVAL;
+  const int rc = calibrate_impl(h, vis, vis_on_device, n_bl, T, k0, l, sbd_ns, mbd_ns, delay_ns, phase_rad, cuda_stream);
+  if (rc != FRBX_OK) settle(h, (cudaStream_t)cuda_stream);
+  return rc;
 }
 
 // ======================================================================================
@@ -1646,10 +1654,9 @@ extern "C" int frbx_batch_info(const frbx_batch *b, frbx_batch_stats *st) {
   return FRBX_OK;
 }
 
-extern "C" int frbx_search_batch(frbx_batch *b, const frbx_scan *scans, int32_t n_scans, const double *dm,
-                                 int32_t n_dm, const int32_t *windows, int32_t n_win, const frbx_params *params,
-                                 frbx_results *results, void *cuda_stream) {
-  if (!b) return FRBX_EINVAL;
+static int search_batch_impl(frbx_batch *b, const frbx_scan *scans, int32_t n_scans, const double *dm, int32_t n_dm,
+                             const int32_t *windows, int32_t n_win, const frbx_params *params, frbx_results *results,
+                             void *cuda_stream) {
   b->err.clear();
   b->launches = 0;
   cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -2094,4 +2101,15 @@ extern "C" int frbx_search_batch(frbx_batch *b, const frbx_scan *scans, int32_t 
   }
   if (trunc) return bfail(b, FRBX_ETRUNC, "an output array was too small");
   return FRBX_OK;
+}
+
+extern "C" int frbx_search_batch(frbx_batch *b, const frbx_scan *scans, int32_t n_scans, const double *dm,
+                                 int32_t n_dm, const int32_t *windows, int32_t n_win, const frbx_params *params,
+                                 frbx_results *results, void *cuda_stream) {
+  if (!b) return FRBX_EINVAL;
+  const int rc = search_batch_impl(b, scans, n_scans, dm, n_dm, windows, n_win, params, results, cuda_stream);
+  if (rc != FRBX_OK && rc != FRBX_ETRUNC && scans && n_scans <= 4096)  // shift tables and fits may be queued
+    for (int32_t i = 0; i < n_scans; ++i)
+      if (scans[i].setup) settle(scans[i].setup, (cudaStream_t)cuda_stream);
+  return rc;
 }
