@@ -415,6 +415,7 @@ int frbx_calibrate(frbx_handle *h, const void *vis, int32_t vis_on_device, int32
  * tile of each setup is chosen by timing candidates on a sample the first time a setup shape
  * is seen by the batch object: 32, 64, 128 APs for the per-segment fit (a stretch of its work
  * items), 512, 1024, 2048 APs for the window tree (one chunk of the setup's longest scan).
+ * The one-kernel window tree of 16-column grids takes a tile by rule, 128 to 1024 APs.
  * The window tree's results do not depend on its tile.
  * Normalisation, threshold and extraction then run per scan as in frbx_search.
  */
@@ -431,7 +432,8 @@ typedef struct frbx_batch_stats {
   int32_t graph_captures;  /* times the fit graph was (re)captured by this batch object */
   int32_t graph_replays;   /* times it was replayed without capture */
   int32_t n_setups;        /* distinct setups in the last call */
-  int32_t time_tile[16];   /* chosen time tile (APs) per setup, in order of first appearance */
+  int32_t time_tile[16];   /* chosen time tile (APs) per setup, in order of first appearance (by rule, of
+                              the setup's longest scan, where the one-kernel window tree runs) */
   int32_t reserved;
   double fit_ms;           /* device time of the last graph launch (all fits) */
   int64_t launches;        /* kernel launches of the last call (graph kernels counted once) */

@@ -1907,13 +1907,18 @@ static int search_batch_impl(frbx_batch *b, const frbx_scan *scans, int32_t n_sc
         if (plan[(size_t)i].setup == (int)g && (i_g < 0 || scans[i].T > scans[i_g].T)) i_g = i;
       float best_ms = 1e30f;
       int best_tt = kTreeTT;
+      bool measured = false;
       for (int TT : kTreeTuneTT) {
         if (i_g < 0) break;
         const FitArgs a = tree_args(i_g);
         TreeRun r;
         plan_tree(h, a, tree_lev[g], windows, n_win, dkm[g], scans[i_g].n_bl, scans[i_g].T, n_dm, a.win_off, a.S_tot,
                   tree_budget(h), tree_tc[g] != 0 ? 0 : -1, &r, TT);
-        if (r.ser.empty() || r.t.fused) break;  // the fused kernel takes a tile of its own
+        if (r.ser.empty()) break;
+        if (r.t.fused) {  // the one-kernel tree takes a tile of its own: nothing to measure
+          best_tt = r.t.TT;
+          break;
+        }
         r.ser.resize(std::min(r.ser.size(), r.chunk));
         if (ensure(h, h->ytree, r.need()) != cudaSuccess || tree_prepare(h) != FRBX_OK) {
           cudaGetLastError();
@@ -1934,12 +1939,13 @@ static int search_batch_impl(frbx_batch *b, const frbx_scan *scans, int32_t n_sc
           FRBX_BCK(b, cudaEventElapsedTime(&ms, b->e0, b->e1));
           ms_min = std::min(ms_min, ms);
         }
+        measured = true;
         if (ms_min < best_ms) {
           best_ms = ms_min;
           best_tt = TT;
         }
       }
-      b->tuned_tt[tkey] = best_tt;
+      if (measured) b->tuned_tt[tkey] = best_tt;
       b->last_tt[g] = best_tt;
     }
     for (int i = 0; i < n_scans; ++i) {

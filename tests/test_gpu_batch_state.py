@@ -1,5 +1,6 @@
-"""What a batch object keeps between calls: the captured graph when the DM trials that leave an AP change.
-And calls, of a batch or of one setup, that fail while work is queued."""
+"""What a batch object keeps between calls and reports: the captured graph when the DM trials that leave an AP change,
+the time tile of setups fitted by the one-kernel window tree, and calls, of a batch or of one setup, that fail
+while work is queued."""
 import numpy as np
 import pytest
 
@@ -30,6 +31,19 @@ def test_more_trials_that_leave_an_ap(frbx, make):  # noqa: F811
                 _same(o, ref.search(v, dms, [2, 4, 8], want_series=True, want_events=True))
         b.search([(h, v) for v in vis], lists[-1], [2, 4, 8])
         assert b.info()["graph_captures"] == len(lists)
+
+
+def test_time_tile_of_the_one_kernel_tree(frbx):  # noqa: F811
+    """Few series of a scan: k_tree16 takes its smallest tile, 128 APs, and that is what is reported."""
+    wl = synth.make_small(T=1500, n_bl=2, dms=[0.0, 10.0])
+    wl.pulses = []
+    h = frbx.Handle.from_workload(wl)
+    v = to_dev(synth.generate(wl))
+    with frbx.Batch() as b:
+        for _ in range(2):
+            b.search([(h, v)], wl.dms, [2, 4])
+            assert b.info()["time_tile"] == [128]
+        assert b.info()["graph_captures"] == 1 and b.info()["graph_replays"] == 1
 
 
 def test_failed_call_returns_after_its_work(frbx):  # noqa: F811
