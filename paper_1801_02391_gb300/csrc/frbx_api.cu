@@ -381,16 +381,13 @@ int frbx_create(const frbx_setup *s, frbx_handle **out) {
     }
     h->b_bytes8 = KA8 * rows * 128;
   }
-  // window-tree tensor-core fit: per block of 48 or 32 MBD columns q (tree_mma_cols), the DFT rows
-  // (Re G of the block's q, then Im G) split as W = W_hi + W_lo in BF16, in 128-byte swizzled images; per 64-wide
-  // K atom the hi rows are followed by the lo rows
-  std::vector<uint16_t> wtree;
-  std::vector<uint8_t> wtree8;
+  // window-tree tensor-core fit: per block of nq MBD columns q (32, and 48 where tree_mma_wide allows),
+  // the DFT rows (Re G of the block's q, then Im G) split as W = W_hi + W_lo in BF16, in 128-byte swizzled
+  // images; per 64-wide K atom the hi rows are followed by the lo rows.  The E4M3 form has the same rows
+  // rounded once to E4M3, 128 K values per 128-byte row.
+  std::vector<uint16_t> wtree[2];
+  std::vector<uint8_t> wtree8[2];
   if (frbx::tree_mma_supported(h->Ls, h->Lm, N, J)) {
-    const int nq = frbx::tree_mma_cols(h->Lm, N), rows = 2 * nq, n_qb = (h->Lm + nq - 1) / nq;
-    const int KA = (2 * N + 63) / 64, atom = rows * 128;
-    const int wb = 2 * KA * atom;  // bytes per block: per K atom, hi rows then lo rows
-    wtree.assign((size_t)n_qb * wb / 2, 0);
     auto bf16 = [](double v) {
       const float f = (float)v;
       uint32_t u;
@@ -404,49 +401,45 @@ int frbx_create(const frbx_setup *s, frbx_handle **out) {
       std::memcpy(&f, &u, 4);
       return (double)f;
     };
-    auto put = [&](int qb, int lo, int R, int k, uint16_t v) {
-      const size_t off = (size_t)qb * wb + (size_t)(k / 64) * 2 * atom + (size_t)lo * atom + (size_t)(R / 8) * 1024 +
-                         (size_t)(R % 8) * 128 + (size_t)((((k % 64) / 8) ^ (R % 8)) * 16) + (size_t)(k % 8) * 2;
-      wtree[off / 2] = v;
-    };
-    for (int qb = 0; qb < n_qb; ++qb)
-      for (int R = 0; R < rows; ++R) {
-        const int q = qb * nq + (R % nq);
-        const bool im = R >= nq;
-        if (q >= h->Lm) continue;  // the last block's columns past the grid stay zero
-        for (int n = 0; n < N; ++n) {
-          const long long ex = ((long long)h->g[(size_t)n] * q) % h->Lm;
-          const double th = two_pi * (double)ex / (double)h->Lm;
-          const double vr = im ? -std::sin(th) : std::cos(th), vi = im ? std::cos(th) : std::sin(th);
-          const uint16_t rh = bf16(vr), ih = bf16(vi);
-          put(qb, 0, R, n, rh);
-          put(qb, 0, R, N + n, ih);
-          put(qb, 1, R, n, bf16(vr - bf16f(rh)));
-          put(qb, 1, R, N + n, bf16(vi - bf16f(ih)));
-        }
+    // cos and sin of 2 pi ex / Lm (at [ex] and [Lm + ex]) and minus the sine ([2 Lm + ex]), in each format
+    const int Lm = h->Lm;
+    std::vector<uint16_t> hi((size_t)3 * Lm), lo((size_t)3 * Lm);
+    std::vector<uint8_t> e4((size_t)3 * Lm);
+    for (int ex = 0; ex < Lm; ++ex) {
+      const double th = two_pi * (double)ex / (double)Lm, v[3] = {std::cos(th), std::sin(th), -std::sin(th)};
+      for (int k = 0; k < 3; ++k) {
+        const size_t i = (size_t)k * Lm + ex;
+        hi[i] = bf16(v[k]);
+        lo[i] = bf16(v[k] - bf16f(hi[i]));
+        e4[i] = to_e4m3(v[k]);
       }
-    h->wtree_bytes = wb;
-    // the E4M3 form: per block the same rows rounded
-    // once to E4M3, 128 K values per 128-byte row
-    const int KA8 = (2 * N + 127) / 128, wb8 = KA8 * rows * 128;
-    wtree8.assign((size_t)n_qb * wb8, 0);
-    auto put8 = [&](int qb, int R, int k, double v) {
-      const size_t off = (size_t)qb * wb8 + (size_t)(k / 128) * rows * 128 + (size_t)(R / 8) * 1024 +
-                         (size_t)(R % 8) * 128 + (size_t)((((k % 128) / 16) ^ (R % 8)) * 16) + (size_t)(k % 16);
-      wtree8[off] = to_e4m3(v);
-    };
-    for (int qb = 0; qb < n_qb; ++qb)
-      for (int R = 0; R < rows; ++R) {
-        const int q = qb * nq + (R % nq);
-        const bool im = R >= nq;
-        if (q >= h->Lm) continue;  // the last block's columns past the grid stay zero
-        for (int n = 0; n < N; ++n) {
-          const long long ex = ((long long)h->g[(size_t)n] * q) % h->Lm;
-          const double th = two_pi * (double)ex / (double)h->Lm;
-          put8(qb, R, n, im ? -std::sin(th) : std::cos(th));
-          put8(qb, R, N + n, im ? std::cos(th) : std::sin(th));
+    }
+    const int KA = (2 * N + 63) / 64, KA8 = (2 * N + 127) / 128;
+    for (int wide = 0; wide <= (frbx::tree_mma_wide(Lm, N) ? 1 : 0); ++wide) {
+      const int nq = wide ? 48 : 32, rows = 2 * nq, n_qb = (Lm + nq - 1) / nq, atom = rows * 128;
+      const size_t wb = (size_t)2 * KA * atom, wb8 = (size_t)KA8 * atom;  // bytes per block
+      wtree[wide].assign(n_qb * wb / 2, 0);
+      wtree8[wide].assign(n_qb * wb8, 0);
+      for (int qb = 0; qb < n_qb; ++qb)
+        for (int R = 0; R < rows; ++R) {
+          const int q = qb * nq + (R % nq);
+          if (q >= Lm) continue;  // the last block's columns past the grid stay zero
+          const size_t row = (size_t)(R / 8) * 1024 + (size_t)(R % 8) * 128;
+          auto put = [&](int k, size_t i) {
+            const size_t off = qb * wb + (size_t)(k / 64) * 2 * atom + row + (size_t)((((k % 64) / 8) ^ (R % 8)) * 16) +
+                               (size_t)(k % 8) * 2;
+            wtree[wide][off / 2] = hi[i];
+            wtree[wide][(off + atom) / 2] = lo[i];
+            wtree8[wide][qb * wb8 + (size_t)(k / 128) * atom + row + (size_t)((((k % 128) / 16) ^ (R % 8)) * 16) +
+                         (size_t)(k % 16)] = e4[i];
+          };
+          for (int n = 0; n < N; ++n) {
+            const size_t ex = (size_t)(((long long)h->g[(size_t)n] * q) % Lm);
+            put(n, R < nq ? ex : 2 * Lm + ex);  // Re: cos, sin; Im: -sin, cos
+            put(N + n, R < nq ? Lm + ex : ex);
+          }
         }
-      }
+    }
   }
   cudaError_t e = cudaGetDevice(&h->device);
   if (e == cudaSuccess) e = upload(&h->d_f, h->f);
@@ -463,8 +456,10 @@ int frbx_create(const frbx_setup *s, frbx_handle **out) {
   if (e == cudaSuccess) e = upload(&h->d_tree_slot, tree_slot);
   if (e == cudaSuccess && !bimg.empty()) e = upload((uint16_t **)&h->d_bimg, bimg);
   if (e == cudaSuccess && !bimg8.empty()) e = upload((uint8_t **)&h->d_bimg8, bimg8);
-  if (e == cudaSuccess && !wtree.empty()) e = upload((uint16_t **)&h->d_wtree, wtree);
-  if (e == cudaSuccess && !wtree8.empty()) e = upload((uint8_t **)&h->d_wtree8, wtree8);
+  for (int w = 0; w < 2 && e == cudaSuccess; ++w) {
+    if (!wtree[w].empty()) e = upload((uint16_t **)&h->d_wtree[w], wtree[w]);
+    if (e == cudaSuccess && !wtree8[w].empty()) e = upload((uint8_t **)&h->d_wtree8[w], wtree8[w]);
+  }
   if (e == cudaSuccess) {
     std::call_once(g_const_once, frbx::set_fft_constants);
     e = cudaGetLastError();
@@ -483,7 +478,7 @@ void frbx_destroy(frbx_handle *h) {
   if (!h) return;
   void *ptrs[] = {h->d_f,      h->d_f0,     h->d_pt,    h->d_wrot, h->d_tw_s, h->d_tw_m,     h->d_g,
                   h->d_sbd_tw, h->d_mbd_tw, h->d_slot, h->d_bimg, h->d_tree_tw, h->d_tree_slot, h->d_bimg8,
-                  h->d_wtree,  h->d_wtree8};
+                  h->d_wtree[0], h->d_wtree[1], h->d_wtree8[0], h->d_wtree8[1]};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   for (cudaEvent_t e : h->ev)
@@ -794,20 +789,73 @@ struct TreeRun {
 // with a +-64 ns window: 37.0 -> 32.2 ms.  (Whole tiles gain nothing from it: short last tiles
 // fill the ends of the rounds.)
 constexpr int kCtaAps = 12;
-int packed_time_tile(int t_max, int pack, int n_s, int n_qb, int lmax) {
+int packed_time_tile(int t_max, int pack, int n_s, int n_qb, int lmax, long long *cost) {
   const long long sms = frbx::sm_count();
-  long long best = INT64_MAX;
   int tile = 64;
+  *cost = INT64_MAX;
   for (int ng = 1;; ++ng) {
     const int tt = (int)(((long long)t_max + 64LL * ng * pack - 1) / (64LL * ng * pack)) * 64;
     if (ng > 1 && tt < 256) break;
-    const long long rounds = ((long long)n_s * n_qb * ng + sms - 1) / sms, cost = rounds * (tt + lmax - 1 + kCtaAps);
-    if (cost < best) {
-      best = cost;
+    const long long rounds = ((long long)n_s * n_qb * ng + sms - 1) / sms, c = rounds * (tt + lmax - 1 + kCtaAps);
+    if (c < *cost) {
+      *cost = c;
       tile = tt;
     }
   }
   return tile;
+}
+
+// AP step of the form with 48 columns (three epilogue warpgroups), in percent of the 32-column one's, both
+// with one CTA per SM.  Measured on 1000 APs of one series (8000 with packed windows), where the longer step
+// is all of the difference: whole grid 644 -> 779 us, without one-AP windows 607 -> 673, with these
+// alone 646 -> 638, one BF16 product 597 -> 764, E4M3 599 -> 722; delay windows of eight
+// pieces 540 -> 574 us (BF16 445 -> 517), four 331 -> 362, two 243 -> 314, one 785 -> 998.
+int wide_step(const frbx::TreeArgs &t, bool full) {
+  if (!full) return t.pack < 4 ? 128 : t.form == 1 ? 117 : 108;
+  if (t.nlev == 0) return 99;
+  return t.form == 1 ? 127 : t.form == 0 && t.emit_w[0] < 0 ? 111 : 120;
+}
+
+// Column blocks, and with TT <= 0 the tile of packed delay windows, of the MBD passes of n_s series (their chunks'
+// launches follow one another without a gap).  Blocks of 48 columns issue better: a full GPU takes 11 of
+// them in the time of 13 of the 16 blocks of 32 that the four-band grid has.  Where they end in as many
+// rounds of CTAs either way, the shorter step of 32 columns wins: 1 series x 4 DM trials x 1500 APs (88 or
+// 128 CTAs on 152 SMs) 1.31 -> 1.19 ms.
+void plan_blocks(const frbx_handle *h, frbx::TreeArgs *t, bool full, int n_s, int t_max, int TT) {
+  const int lmax = 1 << t->nlev;
+  const bool wide_ok = h->d_wtree[1] != nullptr;
+  long long best = INT64_MAX;
+  int cols = 32, tile = t->TT;
+  for (int wide = wide_ok ? 1 : 0; wide >= 0; --wide) {
+    const int nq = wide ? 48 : 32, n_qb = (t->Lm + nq - 1) / nq;
+    int active = 0;  // blocks that hold a searched column
+    for (int b = 0; b < n_qb; ++b) {
+      bool on = false;
+      for (int q = b * nq; q < std::min(t->Lm, (b + 1) * nq); ++q) on |= ((q - t->q_lo) & (t->Lm - 1)) < t->q_len;
+      active += on;
+    }
+    long long cost;
+    int tt = t->TT;
+    if (TT <= 0 && t->pack > 1) {
+      tt = packed_time_tile(t_max, t->pack, n_s, active, lmax, &cost);
+    } else {
+      const long long n_tt = (t_max + tt - 1) / tt, ctas = (n_tt + t->pack - 1) / t->pack * active * n_s;
+      cost = (ctas + frbx::sm_count() - 1) / frbx::sm_count() * (std::min(tt, t_max) + lmax - 1 + kCtaAps);
+    }
+    cost *= wide ? wide_step(*t, full) : 100;
+    if (cost < best) {
+      best = cost;
+      cols = nq;
+      tile = tt;
+    }
+  }
+  t->TT = tile;
+  t->n_tt = (t->T + t->TT - 1) / t->TT;
+  t->n_tg = (t->n_tt + t->pack - 1) / t->pack;
+  t->cols = cols;
+  t->n_qb = (t->Lm + cols - 1) / cols;
+  t->w_bytes = frbx::tree_mma_w_bytes(t->form, cols, h->N);
+  t->wimg = (const unsigned char *)(t->form == 2 ? h->d_wtree8 : h->d_wtree)[cols == 48];
 }
 
 // Host planning: kernel arguments, series list and chunk size for `budget` bytes per set.
@@ -857,8 +905,6 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
     t.KA = form == 2 ? (2 * h->N + 127) / 128 : (2 * h->N + 63) / 64;
     t.k8_steps = (2 * h->N + 31) / 32;
     t.tile_bytes = frbx::tree_mma_tile_bytes(form, h->N);
-    t.wimg = (const unsigned char *)(form == 2 ? h->d_wtree8 : h->d_wtree);
-    t.w_bytes = frbx::tree_mma_w_bytes(form, h->Lm, h->N);
     // delay windows: rotate the SBD rows so the searched ones come first (in groups of 8)
     t.rot = r->full ? 0 : (a.m_lo & ~7);
     // rows searched after the rotation: [m_lo mod 8, m_lo mod 8 + m_len)
@@ -866,8 +912,6 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
     t.pack = rows <= 16 ? 8 : rows <= 32 ? 4 : rows <= 64 ? 2 : 1;
     t.prow = 128 / t.pack;
     t.piece_bytes = t.tile_bytes / t.pack;
-    const int cols = frbx::tree_mma_cols(h->Lm, h->N);
-    t.n_qb = (h->Lm + cols - 1) / cols;
     t.log2Lm = a.log2Lm;
     t.err = (int *)h->errflag.p;
     t.timeout = wait_cycles(h);
@@ -898,12 +942,8 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
   const size_t most = copying && mma ? std::max<size_t>(1, all / (size_t)n_bl) : all;
   r->chunk = t.fused ? all : std::max<size_t>(1, std::min(most, budget / per));
   if (mma) {
-    if (TT <= 0 && t.pack > 1 && !r->ser.empty()) {
-      const int t_max = T - *std::min_element(dkm.begin(), dkm.end());
-      t.TT = packed_time_tile(t_max, t.pack, (int)std::min(r->chunk, r->ser.size()), t.n_qb, 1 << nlev);
-      t.n_tt = (T + t.TT - 1) / t.TT;
-    }
-    t.n_tg = (t.n_tt + t.pack - 1) / t.pack;
+    const int t_max = r->ser.empty() ? 1 : T - *std::min_element(dkm.begin(), dkm.end());
+    plan_blocks(h, &t, r->full, (int)all, t_max, TT);
   }
   r->sc_off = (sizeof(float2) * t.y_series * r->chunk + 255) & ~(size_t)255;
   r->y_bytes = r->sc_off + ((sc_per * r->chunk + 255) & ~(size_t)255);
@@ -1305,7 +1345,7 @@ static int search_impl(frbx_handle *h, const void *vis, int32_t vis_on_device, i
   int nlev = 0;
   const bool tree_ok = frbx::tree_supported(h->Ls, h->Lm, h->N, h->J, h->tree_s16, windows, n_win, &nlev);
   // tensor-core window tree: kernel 6 (split BF16, FP32-equivalent), 7 (BF16), 8 (E4M3)
-  const bool tree_tc_shape = tree_ok && h->d_wtree && frbx::tree_mma_supported(h->Ls, h->Lm, h->N, h->J);
+  const bool tree_tc_shape = tree_ok && h->d_wtree[0] && frbx::tree_mma_supported(h->Ls, h->Lm, h->N, h->J);
   const int tc_form = p.kernel == 7 ? 1 : p.kernel == 8 ? 2 : 0;
   const bool tree_tc = tree_tc_shape && frbx::tree_mma_fits(tc_form, h->Lm, h->N, nlev);
   if ((p.kernel == 4 && !tree_ok) || (p.kernel >= 6 && !tree_tc))
@@ -1706,7 +1746,7 @@ static int search_batch_impl(frbx_batch *b, const frbx_scan *scans, int32_t n_sc
     int nlev = 0;
     const bool ok = frbx::tree_supported(h->Ls, h->Lm, h->N, h->J, h->tree_s16, windows, n_win, &nlev);
     const FitArgs &ag = fa[g];
-    const bool tc_ok = ok && h->d_wtree && frbx::tree_mma_supported(h->Ls, h->Lm, h->N, h->J) &&
+    const bool tc_ok = ok && h->d_wtree[0] && frbx::tree_mma_supported(h->Ls, h->Lm, h->N, h->J) &&
                        frbx::tree_mma_fits(0, h->Lm, h->N, nlev);
     (void)ag;
     if ((p.kernel == 4 && !ok) || (p.kernel == 6 && !tc_ok))

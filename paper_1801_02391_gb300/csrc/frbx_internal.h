@@ -181,8 +181,9 @@ struct TreeArgs {
   size_t yt_series;        // bytes per series in Yt
   int KA;                  // 64-wide K atoms per tile row (K = 2N)
   int tile_bytes;          // one AP: hi tile then lo tile, 2 KA 16 KB
-  const unsigned char *wimg;  // [n_qb][KA][hi | lo][2 tree_mma_cols() rows x 128 B]
-  int w_bytes;             // per block of tree_mma_cols() columns q
+  const unsigned char *wimg;  // [n_qb][KA][hi | lo][2 cols rows x 128 B]
+  int w_bytes;             // per block of cols columns q
+  int cols;                // columns q per CTA: 48 or 32
   int n_qb;                // column blocks
   int log2Lm;
   int *err;                // set to FRBX_ETIMEOUT when a bounded wait of k_tree_mma gives up
@@ -202,10 +203,10 @@ struct TreeArgs {
   int n_sanc;              // window-tree anchor levels of k_tree_mma in shared memory (set by its launcher)
 };
 bool tree_mma_supported(int Ls, int Lm, int N, int J);
-int tree_mma_cols(int Lm, int N);  // MBD columns q per CTA of k_tree_mma
+bool tree_mma_wide(int Lm, int N);  // k_tree_mma can take 48 MBD columns per CTA, not only 32
 bool tree_mma_fits(int form, int Lm, int N, int nlev);  // shared memory holds W, the A ring and the deep anchors
 int tree_mma_tile_bytes(int form, int N);        // one AP's A operand in its shared-memory image
-int tree_mma_w_bytes(int form, int Lm, int N);   // the DFT operand of one column block
+int tree_mma_w_bytes(int form, int cols, int N); // the DFT operand of one column block
 cudaError_t launch_tree_mma(const TreeArgs &t, bool full, cudaStream_t st, int64_t *launches);
 bool tree_supported(int Ls, int Lm, int N, int J, int s16, const int *windows, int n_win, int *nlev);
 int tree_rows_per_block(int Ls, int Lm);  // SBD rows per k_tree_mbd CTA
@@ -304,9 +305,8 @@ struct frbx_handle {
   int tree_tensor = 0;               // 1: its MBD pass ran on the tensor cores (k_tree_mma)
   void *d_bimg = nullptr;  // BF16 DFT matrix image for the tensor-core fit (if supported)
   void *d_bimg8 = nullptr;  // the same matrix in E4M3
-  void *d_wtree = nullptr;  // window-tree tensor-core fit: split-BF16 DFT blocks of tree_mma_cols() q
-  void *d_wtree8 = nullptr; // the same blocks in E4M3 (kernel 8)
-  int wtree_bytes = 0;      // per block
+  void *d_wtree[2] = {nullptr, nullptr};  // window-tree tensor-core fit: split-BF16 DFT blocks of 32 and of 48 q
+  void *d_wtree8[2] = {nullptr, nullptr}; // the same blocks in E4M3 (kernel 8)
   int b_bytes = 0, b_bytes8 = 0, b_atom_bytes = 0, KA = 0, NC = 0;
   int *d_g = nullptr, *d_slot = nullptr;
   // scratch, grown on demand

@@ -734,10 +734,11 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
 
 // Column blocks of 48 (three epilogue warpgroups) where one 64-wide K atom holds the operand: three
 // epilogue warps per sub-partition instead of two hide more of each warp's chain, and an A tile is
-// read by Lm / 48 CTAs instead of Lm / 32.  Blocks of 32 where 48 would leave a third of the block
+// read by Lm / 48 CTAs instead of Lm / 32.  Not where 48 would leave a third of the block
 // empty (Lm 32 and 64), or where 2N > 64 doubles the tiles and the operand, which beside 48-column
-// anchors in shared memory would leave no room for two ring buffers.
-int tree_mma_cols(int Lm, int N) { return 2 * N <= 64 && Lm > 64 ? 48 : 32; }
+// anchors in shared memory would leave no room for two ring buffers.  plan_blocks (frbx_api.cu) chooses
+// by launch: small ones take 32.
+bool tree_mma_wide(int Lm, int N) { return 2 * N <= 64 && Lm > 64; }
 
 bool tree_mma_supported(int Ls, int Lm, int N, int J) {
   return Ls == tc::kRows && J <= Ls && Lm % 32 == 0 && 2 * N <= 128;
@@ -746,11 +747,11 @@ bool tree_mma_supported(int Ls, int Lm, int N, int J) {
 bool tree_mma_fits(int form, int Lm, int N, int nlev) {
   int nb, ns;
   return form >= kFormSplit && form <= kFormFp8 && nlev >= 0 && nlev <= kTmMaxLev &&
-         tm_plan(form, N, tree_mma_cols(Lm, N) / kQ, nlev, &nb, &ns);
+         tm_plan(form, N, 2, nlev, &nb, &ns) && (!tree_mma_wide(Lm, N) || tm_plan(form, N, 3, nlev, &nb, &ns));
 }
 
 int tree_mma_tile_bytes(int form, int N) { return tm_tile_bytes(form, N); }
-int tree_mma_w_bytes(int form, int Lm, int N) { return tm_w_bytes(form, N, tree_mma_cols(Lm, N) / kQ); }
+int tree_mma_w_bytes(int form, int cols, int N) { return tm_w_bytes(form, N, cols / kQ); }
 
 template <int kParts, int kForm, bool kFull, bool kOne = true>
 static cudaError_t launch_tm_one(const TreeArgs &u, unsigned nb, size_t smem, cudaStream_t st) {
@@ -783,8 +784,8 @@ static cudaError_t launch_tm(const TreeArgs &u, bool full, unsigned g, size_t sm
 }
 
 cudaError_t launch_tree_mma(const TreeArgs &t, bool full, cudaStream_t st, int64_t *launches) {
-  const int cols = tree_mma_cols(t.Lm, t.N), parts = cols / kQ;
-  if (t.nlev < 0 || t.nlev > kTmMaxLev || t.form < kFormSplit || t.form > kFormFp8 || t.KA != tm_katoms(t.form, t.N) ||
+  const int cols = t.cols, parts = cols / kQ;
+  if (!(cols == 32 || (cols == 48 && tree_mma_wide(t.Lm, t.N))) || t.nlev < 0 || t.nlev > kTmMaxLev || t.form < kFormSplit || t.form > kFormFp8 || t.KA != tm_katoms(t.form, t.N) ||
       t.w_bytes != tm_w_bytes(t.form, t.N, parts) || t.tile_bytes != tm_tile_bytes(t.form, t.N) ||
       t.n_qb != (t.Lm + cols - 1) / cols ||
       (t.form == kFormFp8 && (!t.ascale || t.k8_steps != (2 * t.N + 31) / 32)) || (full && t.rot != 0) ||
