@@ -937,9 +937,17 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
   const size_t sc_per = form == 2 ? sizeof(float) * (size_t)T : 0;
   const size_t per = sizeof(float2) * t.y_series + sc_per + anc_per;
   const size_t all = std::max<size_t>(r->ser.size(), 1);
-  // a cube still being copied from the host, one baseline after another: no chunk waits for more than
-  // one (a search of 2 baselines x 2411 APs from pinned memory 6.27 -> 6.11 ms)
-  const size_t most = copying && mma ? std::max<size_t>(1, all / (size_t)n_bl) : all;
+  // a cube still being copied from the host, one baseline after another: a chunk waits for no more of them
+  // than fill the SMs with CTAs, in chunks of equal length (2 baselines x 16 DM trials x 2411 APs from pinned
+  // memory in one chunk 6.3, in two 6.15 ms; 15 x 2 x 300 in one 1.55, in three 1.29, in fifteen 2.94 ms;
+  // with room for two rounds of CTAs a chunk 1.46 ms)
+  size_t most = all;
+  if (copying && mma) {
+    const long long wide = h->d_wtree[1] ? 48 : 32, n_tg = (t.n_tt + t.pack - 1) / t.pack;
+    const long long per_bl = std::max<long long>(1, (long long)(all / (size_t)n_bl) * ((h->Lm + wide - 1) / wide) * n_tg);
+    const long long group = std::max<long long>(1, frbx::sm_count() / per_bl), n_ch = (n_bl + group - 1) / group;
+    most = std::max<size_t>(1, all / (size_t)n_bl * (size_t)((n_bl + n_ch - 1) / n_ch));
+  }
   r->chunk = t.fused ? all : std::max<size_t>(1, std::min(most, budget / per));
   if (mma) {
     const int t_max = r->ser.empty() ? 1 : T - *std::min_element(dkm.begin(), dkm.end());
