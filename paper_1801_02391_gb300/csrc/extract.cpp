@@ -5,7 +5,7 @@
 // is the first group (in creation order) holding a member whose [k0, k0 + l) overlaps
 // mine", answered from a per-AP array of the smallest group id covering that AP.  Steps b to d of
 // one (series, DM trial) depend on its own events only, so event lists are split there
-// across host threads; the DM merge and cross-matching see the pulses of all, which are few.
+// across host threads, and the DM merge between series; cross-matching sees the merged pulses of all.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -142,64 +142,88 @@ void extract_events(const ExtractConfig &cfg, const CircleTable &circle, const f
 }
 
 // Sec. 5.3: per series, one pulse per overlap group across DM trials, the one of highest power.
-// pulses: sorted by series, DM trials ascending.
-void merge_dm(const ExtractConfig &cfg, const std::vector<Pulse> &pulses, std::vector<Pulse> *merged) {
+// p[0, n): sorted by series, DM trials ascending.
+void merge_dm(const ExtractConfig &cfg, const Pulse *p, size_t n, std::vector<Pulse> *merged) {
   Grouper gm(cfg.T);
   std::vector<size_t> best_of;
-  for (size_t i = 0; i < pulses.size();) {
-    const int s = pulses[i].series;
+  for (size_t i = 0; i < n;) {
+    const int s = p[i].series;
     gm.reset();
     best_of.clear();
-    for (; i < pulses.size() && pulses[i].series == s; ++i) {
-      const size_t g = (size_t)gm.insert(pulses[i].k0, pulses[i].l);
+    for (; i < n && p[i].series == s; ++i) {
+      const size_t g = (size_t)gm.insert(p[i].k0, p[i].l);
       if (g == best_of.size()) best_of.push_back(i);
-      else if (pulses[i].p > pulses[best_of[g]].p) best_of[g] = i;
+      else if (p[i].p > p[best_of[g]].p) best_of[g] = i;
     }
-    for (size_t k : best_of) merged->push_back(pulses[k]);
+    for (size_t k : best_of) merged->push_back(p[k]);
   }
 }
 
-// Events per host thread: a thread costs about 20 us to start, an event about 50 ns.
+// Events (pulses, in the DM merge) per host thread: a thread costs about 20 us to start, an event about 50 ns.
 constexpr int64_t kEventsPerThread = 2000;
 
-}  // namespace
-
-// Contiguous runs of (series, DM trial)s go to host threads, balanced by event count, the last one to
-// the calling thread, and their pulses are concatenated in order: the same output as one pass.
-void extract_pulses(const ExtractConfig &cfg, const frbx_event *ev, int64_t n_ev, int n_series,
-                    bool use_mbd, std::vector<Pulse> *pre_merge, std::vector<Pulse> *merged) {
-  (void)n_series;
-  const CircleTable circle(use_mbd ? cfg.Lm : 0);
+// Cuts [0, n) into contiguous parts of about equal length, at most one per kEventsPerThread items and per host
+// thread, none between items i - 1 and i that belong together(i), calls parts(their number) and runs
+// run(part, begin, end) for each, the last one on the calling thread.
+template <class Together, class Parts, class Run>
+void on_threads(int64_t n, Together together, Parts parts, Run run) {
   const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
-  const int n_th = (int)std::max<int64_t>(1, std::min<int64_t>({n_ev / kEventsPerThread, (int64_t)hw, (int64_t)32}));
-  // part t starts at the first event of a (series, DM trial) at or after t n_ev / n_th
-  std::vector<int64_t> cut((size_t)n_th + 1, n_ev);
+  const int n_th = (int)std::max<int64_t>(1, std::min<int64_t>({n / kEventsPerThread, (int64_t)hw, (int64_t)32}));
+  parts((size_t)n_th);
+  std::vector<int64_t> cut((size_t)n_th + 1, n);
   cut[0] = 0;
   for (int t = 1; t < n_th; ++t) {
-    int64_t i = std::max(cut[(size_t)t - 1], n_ev * t / n_th);
-    while (i > 0 && i < n_ev && ev[i].series == ev[i - 1].series && ev[i].dm_idx == ev[i - 1].dm_idx) ++i;
+    int64_t i = std::max(cut[(size_t)t - 1], n * t / n_th);
+    while (i > 0 && i < n && together(i)) ++i;
     cut[(size_t)t] = i;
   }
-  std::vector<std::vector<Pulse>> part((size_t)n_th);
-  auto run = [&](int t) {
-    const int64_t e0 = cut[(size_t)t], e1 = cut[(size_t)t + 1];
-    if (e0 < e1) extract_events(cfg, circle, ev + e0, e1 - e0, use_mbd, &part[(size_t)t]);
+  auto part = [&](int t) {
+    if (cut[(size_t)t] < cut[(size_t)t + 1]) run((size_t)t, cut[(size_t)t], cut[(size_t)t + 1]);
   };
   std::vector<std::thread> th;
   th.reserve((size_t)n_th);
   for (int t = 0; t + 1 < n_th; ++t) {
     try {
-      th.emplace_back(run, t);
+      th.emplace_back(part, t);
     } catch (...) {  // no thread to be had: this part runs here (no exception crosses the C ABI)
-      run(t);
+      part(t);
     }
   }
-  run(n_th - 1);
+  part(n_th - 1);
   for (auto &x : th) x.join();
+}
+
+void append(const std::vector<std::vector<Pulse>> &parts, std::vector<Pulse> *out) {
+  size_t n = out->size();
+  for (const auto &p : parts) n += p.size();
+  out->reserve(n);
+  for (const auto &p : parts) out->insert(out->end(), p.begin(), p.end());
+}
+
+}  // namespace
+
+// Runs of (series, DM trial)s go to host threads, then, for the DM merge of their pulses, runs of series; the
+// parts' pulses are concatenated in order: the same output as one pass.  Where one window is enough, nearly
+// every event is a pulse: 64 series x 16 DM trials with 464000 of them 34.6 -> 8.4 ms on 16 cores against the
+// merge on one thread, 15.6 ms with both steps split by series.
+void extract_pulses(const ExtractConfig &cfg, const frbx_event *ev, int64_t n_ev, int n_series,
+                    bool use_mbd, std::vector<Pulse> *pre_merge, std::vector<Pulse> *merged) {
+  (void)n_series;
+  const CircleTable circle(use_mbd ? cfg.Lm : 0);
+  std::vector<std::vector<Pulse>> part;
+  on_threads(
+      n_ev, [&](int64_t i) { return ev[i].series == ev[i - 1].series && ev[i].dm_idx == ev[i - 1].dm_idx; },
+      [&](size_t n) { part.resize(n); },
+      [&](size_t t, int64_t e0, int64_t e1) { extract_events(cfg, circle, ev + e0, e1 - e0, use_mbd, &part[t]); });
   std::vector<Pulse> all = std::move(part[0]);
-  for (int t = 1; t < n_th; ++t) all.insert(all.end(), part[(size_t)t].begin(), part[(size_t)t].end());
-  merge_dm(cfg, all, merged);
-  if (pre_merge) pre_merge->insert(pre_merge->end(), all.begin(), all.end());
+  part[0].clear();
+  append(part, &all);
+  on_threads(
+      (int64_t)all.size(), [&](int64_t i) { return all[(size_t)i].series == all[(size_t)i - 1].series; },
+      [&](size_t n) { part.assign(n, {}); },
+      [&](size_t t, int64_t i0, int64_t i1) { merge_dm(cfg, all.data() + i0, (size_t)(i1 - i0), &part[t]); });
+  append(part, merged);
+  if (pre_merge) *pre_merge = std::move(all);
 }
 
 void cross_match(int T, std::vector<Pulse> *merged, int n_bl, std::vector<GroupOut> *groups) {
