@@ -212,7 +212,10 @@ __device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint64_t ad, uint64_t 
 // rotation).
 // kOne: windows of one AP are searched; without them no AP's own maximum is formed, a sixth of the
 // epilogue's instructions (built for the default product; five scans with windows of 2 to 16 APs: 50.4 -> 46.7 ms).
-template <int kParts, int kForm, bool kFull, bool kOne>
+// kSplit: delay windows of eight pieces, a warp's lanes on two time tiles; an instance of its own, since the other
+// windows pay for the second maximum otherwise (1 series x 4 DM trials x 1500 APs with a
+// +-1 ns MBD window 1.38 -> 1.28 ms).
+template <int kParts, int kForm, bool kFull, bool kOne, bool kSplit>
 __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(const __grid_constant__ TreeArgs t) {
   using Sh = TmShape<kParts>;
   constexpr int kEpi = Sh::kEpi, kMmaWarp = kEpi, kLoadWarp = kEpi + 1, kNQ = Sh::kNQ, kCols = Sh::kCols;
@@ -414,12 +417,12 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
     // this lane's time tile (its piece of the packed operand) and its first AP and AP count; the warp
     // walks n_me APs, those of its first tile (with eight pieces a warp holds two, 16 lanes each, the
     // second of them no longer)
-    const bool split = !kFull && pack == 8;
-    const int qpp = split ? 1 : 4 / pack, my_p = split ? 2 * quarter + (lane >> 4) : quarter / qpp;
-    const int kb_me = tile_kb(my_p), n_mine = tile_n(my_p), n_me = split ? tile_n(2 * quarter) : n_mine;
+    static_assert(!(kFull && kSplit), "whole grids are not packed");
+    const int qpp = kSplit ? 1 : 4 / pack, my_p = kSplit ? 2 * quarter + (lane >> 4) : quarter / qpp;
+    const int kb_me = tile_kb(my_p), n_mine = tile_n(my_p), n_me = kSplit ? tile_n(2 * quarter) : n_mine;
     // this lane's SBD row m (row (quarter mod qpp) 32 + lane of its piece, rotated by t.rot) and
     // its first cell
-    const int m_row = (split ? (lane & 15) + t.rot : (quarter % qpp) * 32 + lane + t.rot) & (t.Ls - 1);
+    const int m_row = (kSplit ? (lane & 15) + t.rot : (quarter % qpp) * 32 + lane + t.rot) & (t.Ls - 1);
     const unsigned idx_base = (unsigned)(m_row * t.Lm + qb * kNQ + kQ * part);
     // delay windows: the lane's row is searched, and which of its kQ cells
     const bool row_on = kFull || (((m_row - t.m_lo) & (t.Ls - 1)) < t.m_len);
@@ -503,11 +506,13 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
     // starting before the tile is never issued)
     unsigned long long *const base0 = keys + woff[0] + kb_me, *const base1 = keys + woff[1] + kb_me,
                               *const base2 = keys + woff[2] + (kb_me >> 1);
-    // (the delay-window form has no registers to spare for them: slots, added to keys at each merge)
+    // (three parts with delay windows, and eight pieces, have no registers to spare for them: slots, added to
+    // keys at each merge)
+    constexpr bool kBase = kFull || (kParts == 2 && !kSplit);
     const int o0 = woff[0] + kb_me, o1 = woff[1] + kb_me, o2 = woff[2] + (kb_me >> 1);
     auto merge = [&](const int e, const int i0, const unsigned tkey, const bool on) {
-      unsigned wmax = __reduce_max_sync(0xffffffffu, !kFull && split && lane >= 16 ? 0u : tkey);
-      if (!kFull && split) {  // each tile's 16 lanes by themselves
+      unsigned wmax = __reduce_max_sync(0xffffffffu, kSplit && lane >= 16 ? 0u : tkey);
+      if (kSplit) {  // each tile's 16 lanes by themselves
         const unsigned hi = __reduce_max_sync(0xffffffffu, lane >= 16 ? tkey : 0u);
         if (lane >= 16) wmax = hi;
       }
@@ -515,7 +520,7 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
       const unsigned idx = idx_base + (31u - (wmax & 63u));
       // slot of the segment: windows of 2^e APs start every 2^(e-1) APs (every AP for e = 0)
       unsigned long long *dst = e > 2    ? keys + woff[e] + ((kb_me + i0) >> (e - 1))
-                                : !kFull ? keys + (e == 0 ? o0 + i0 : e == 1 ? o1 + i0 : o2 + (i0 >> 1))
+                                : !kBase ? keys + (e == 0 ? o0 + i0 : e == 1 ? o1 + i0 : o2 + (i0 >> 1))
                                 : e == 0 ? base0 + i0
                                 : e == 1 ? base1 + i0
                                          : base2 + (i0 >> 1);
@@ -561,7 +566,7 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
           if (i0 < 0 || i0 >= t.TT) em &= ~(1u << e);
         }
       }
-      if (!kFull && i >= n_mine) em = 0u;  // the second tile of the warp has ended
+      if (kSplit && i >= n_mine) em = 0u;  // the second tile of the warp has ended
       tm_wait_ld();
       tm_take(rre, cre);
       tm_take(rim, cim);
@@ -671,7 +676,8 @@ __global__ void __launch_bounds__(TmShape<kParts>::kWarps * 32, 1) k_tree_mma(co
           aim[p] = add2(aim[p], oim[p]);
         }
         if (in_tmem) tm_wait_st();
-        if (__any_sync(0xffffffffu, (em >> e) & 1u)) emit(e, i - (1 << e) + 1, are, aim, (em >> e) & 1u);
+        const bool on = (em >> e) & 1u;  // uniform but for two tiles in a warp
+        if (kSplit ? __any_sync(0xffffffffu, on) : on) emit(e, i - (1 << e) + 1, are, aim, on);
       }
       return true;
     };
@@ -753,10 +759,10 @@ bool tree_mma_fits(int form, int Lm, int N, int nlev) {
 int tree_mma_tile_bytes(int form, int N) { return tm_tile_bytes(form, N); }
 int tree_mma_w_bytes(int form, int cols, int N) { return tm_w_bytes(form, N, cols / kQ); }
 
-template <int kParts, int kForm, bool kFull, bool kOne = true>
+template <int kParts, int kForm, bool kFull, bool kOne = true, bool kSplit = false>
 static cudaError_t launch_tm_one(const TreeArgs &u, unsigned nb, size_t smem, cudaStream_t st) {
   using Sh = TmShape<kParts>;
-  auto kern = k_tree_mma<kParts, kForm, kFull, kOne>;
+  auto kern = k_tree_mma<kParts, kForm, kFull, kOne, kSplit>;
   // the register split inside the kernel assumes the launch allocation of kLaunchRegs per thread
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, kern);
@@ -768,19 +774,19 @@ static cudaError_t launch_tm_one(const TreeArgs &u, unsigned nb, size_t smem, cu
   return cudaGetLastError();
 }
 
+template <int kParts, int kForm, bool kOne = true>
+static cudaError_t launch_tm_form(const TreeArgs &u, bool full, unsigned g, size_t smem, cudaStream_t st) {
+  if (full) return launch_tm_one<kParts, kForm, true, kOne>(u, g, smem, st);
+  return u.pack == 8 ? launch_tm_one<kParts, kForm, false, kOne, true>(u, g, smem, st)
+                     : launch_tm_one<kParts, kForm, false, kOne>(u, g, smem, st);
+}
+
 template <int kParts>
 static cudaError_t launch_tm(const TreeArgs &u, bool full, unsigned g, size_t smem, cudaStream_t st) {
-  if (u.form == kFormSplit && u.emit_w[0] < 0)
-    return full ? launch_tm_one<kParts, kFormSplit, true, false>(u, g, smem, st)
-                : launch_tm_one<kParts, kFormSplit, false, false>(u, g, smem, st);
-  switch (u.form * 2 + (full ? 1 : 0)) {
-    case 0: return launch_tm_one<kParts, kFormSplit, false>(u, g, smem, st);
-    case 1: return launch_tm_one<kParts, kFormSplit, true>(u, g, smem, st);
-    case 2: return launch_tm_one<kParts, kFormBf16, false>(u, g, smem, st);
-    case 3: return launch_tm_one<kParts, kFormBf16, true>(u, g, smem, st);
-    case 4: return launch_tm_one<kParts, kFormFp8, false>(u, g, smem, st);
-    default: return launch_tm_one<kParts, kFormFp8, true>(u, g, smem, st);
-  }
+  if (u.form == kFormFp8) return launch_tm_form<kParts, kFormFp8>(u, full, g, smem, st);
+  if (u.form == kFormBf16) return launch_tm_form<kParts, kFormBf16>(u, full, g, smem, st);
+  return u.emit_w[0] < 0 ? launch_tm_form<kParts, kFormSplit, false>(u, full, g, smem, st)
+                         : launch_tm_form<kParts, kFormSplit>(u, full, g, smem, st);
 }
 
 cudaError_t launch_tree_mma(const TreeArgs &t, bool full, cudaStream_t st, int64_t *launches) {
