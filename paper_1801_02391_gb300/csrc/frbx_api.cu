@@ -909,7 +909,8 @@ void plan_tree(const frbx_handle *h, const FitArgs &a, int nlev, const int32_t *
     t.rot = r->full ? 0 : (a.m_lo & ~7);
     // rows searched after the rotation: [m_lo mod 8, m_lo mod 8 + m_len)
     const int rows = r->full ? h->Ls : (a.m_lo & 7) + a.m_len;
-    t.pack = rows <= 16 ? 8 : rows <= 32 ? 4 : rows <= 64 ? 2 : 1;
+    // (a tile that is given may leave half of eight pieces empty: four of 32 rows then, whose step is shorter)
+    t.pack = rows <= 16 && (TT <= 0 || t.n_tt > 4) ? 8 : rows <= 32 ? 4 : rows <= 64 ? 2 : 1;
     t.prow = 128 / t.pack;
     t.piece_bytes = t.tile_bytes / t.pack;
     t.log2Lm = a.log2Lm;
