@@ -313,14 +313,16 @@ int frbx_extract_events(const frbx_event *events, int64_t n_events, int32_t n_se
  *  [0] shift table (Eq. 1-2)        [1] segment fit kernel (Eq. 3, Eq. 5, Sec. 5.1)
  *  [2] baselines: Eq. 6 + threshold  [3] combinations: sum + Eq. 6 + threshold
  *  [4] host extraction (Sec. 2.4.1 b-d, Sec. 5.3 merge, cross-matching, Sec. 2.4.2)
- *  [5] window-tree fit: device time of its SBD-pass kernels, summed over its chunks
- *  [6] window-tree fit: device time of its MBD-pass kernels (k_tree_mbd or k_tree_mma), summed
- *  [7] window-tree fit: number of chunks (= launches of each of the two kernels)
+ *  [5] window-tree fit: device time of its SBD-pass kernels, summed over its chunks (about 0 where one
+ *      kernel, k_tree16, does both passes)
+ *  [6] window-tree fit: device time of its MBD-pass kernels (k_tree_mbd, k_tree_mma or k_tree16): each
+ *      counts from the end of the one before where two overlap
+ *  [7] window-tree fit: number of chunks (= launches of each of its kernels)
  *  [8] window-tree fit: 1 if its MBD pass ran on the tensor cores (k_tree_mma), else 0
  *  ms_out  [n] out, milliseconds (stages that did not run report 0).
  * Stages [5] and [6] are bracketed by events on the library's own streams (SBD passes on
- * one, MBD passes on the other); the SBD pass of a chunk overlaps the MBD pass of the
- * previous one, so [5] + [6] can exceed [1].
+ * one, MBD passes of even and odd chunks on two others); the SBD pass of a chunk overlaps the MBD
+ * pass of the previous one, so [5] + [6] can exceed [1].
  * Returns the number of values written (min(n, 9)) or FRBX_EINVAL.
  */
 int frbx_last_stage_times(const frbx_handle *h, double *ms_out, int32_t n);
@@ -411,7 +413,7 @@ int frbx_calibrate(frbx_handle *h, const void *vis, int32_t vis_on_device, int32
  * per distinct window layout), whose CTAs claim (scan, baseline, time tile, DM trial) work
  * items from a device counter, so uneven scans load-balance; these launches are captured once
  * into a CUDA graph and replayed while the scans' shapes and buffers stay the same; setups
- * that take the window-tree fit add its two passes per chunk of series to the graph.  The time
+ * that take the window-tree fit add its passes per chunk of series to the graph.  The time
  * tile of each setup is chosen by timing candidates on a sample the first time a setup shape
  * is seen by the batch object: 32, 64, 128 APs for the per-segment fit (a stretch of its work
  * items), 512, 1024, 2048 APs for the window tree (one chunk of the setup's longest scan).
@@ -471,7 +473,8 @@ int64_t frbx_last_launch_count(const frbx_handle *h);
  *                     flight before a CTA exits keep the 2e9 limit, so no CTA leaves work behind.
  *  scratch_cap_bytes  cap on the device scratch the handle holds (the buffers it grows on demand;
  *                     the constant tables of frbx_create are not counted).  Default: no cap.  A
- *                     call that would grow the scratch past the cap returns FRBX_ENOMEM.
+ *                     call that would grow the scratch past the cap returns FRBX_ENOMEM (the
+ *                     normalisation's hit mask, a bit per slot, is given up first).
  *  hold_producers     test aid, 0 = off.  The producer roles of the tensor-core kernels issue
  *                     nothing, so the consumers' bounded waits run out: the call returns
  *                     FRBX_ETIMEOUT without any fault, nothing is left in flight and the handle

@@ -781,12 +781,12 @@ struct TreeRun {
   size_t need() const { return 2 * (y_bytes + a_bytes); }  // two buffer sets: chunks alternate
 };
 
-// Time tile of a tensor-core MBD launch of n_s series with packed delay windows: one CTA per SM walks pack
-// tiles side by side, so a launch takes rounds(CTAs / SMs) times the APs of a tile, the lmax - 1 trailing
-// APs it repeats and about kCtaAps APs' time of setup.  Tiles of equal length (t_max: APs of the longest
-// sweep-free stretch), a multiple of pack of them, in the number that makes this least.  Fixed tiles left
-// pieces empty: 9973 APs in 2048-AP tiles are five, so the second group of four held one.  32 x 3 series
-// with a +-64 ns window: 37.0 -> 32.2 ms.  (Whole tiles gain nothing from it: short last tiles
+// Time tile of the tensor-core MBD passes of n_s series with packed delay windows, n_qb column blocks each: one
+// CTA per SM walks pack tiles side by side, so a launch takes rounds(CTAs / SMs) times the APs of a tile, the
+// lmax - 1 trailing APs it repeats and about kCtaAps APs' time of setup.  Tiles of equal length (t_max: APs of
+// the longest sweep-free stretch), a multiple of pack of them, in the number that makes this least (*cost).
+// Fixed tiles left pieces empty: 9973 APs in 2048-AP tiles are five, so the second group of four held one.
+// 32 x 3 series with a +-64 ns window: 37.0 -> 31.6 ms.  (Whole tiles gain nothing from it: short last tiles
 // fill the ends of the rounds.)
 constexpr int kCtaAps = 12;
 int packed_time_tile(int t_max, int pack, int n_s, int n_qb, int lmax, long long *cost) {
@@ -807,13 +807,13 @@ int packed_time_tile(int t_max, int pack, int n_s, int n_qb, int lmax, long long
 
 // AP step of the form with 48 columns (three epilogue warpgroups), in percent of the 32-column one's, both
 // with one CTA per SM.  Measured on 1000 APs of one series (8000 with packed windows), where the longer step
-// is all of the difference: whole grid 644 -> 779 us, without one-AP windows 607 -> 673, with these
-// alone 646 -> 638, one BF16 product 597 -> 764, E4M3 599 -> 722; delay windows of eight
-// pieces 540 -> 574 us (BF16 445 -> 517), four 331 -> 362, two 243 -> 314, one 785 -> 998.
+// is all of the difference: whole grid 646 -> 781 us, without one-AP windows 607 -> 675, with these
+// alone 646 -> 638, one BF16 product 593 -> 765, E4M3 599 -> 724; delay windows of eight
+// pieces 544 -> 574 us (BF16 450 -> 517), four 329 -> 353, two 230 -> 282, one 753 -> 912.
 int wide_step(const frbx::TreeArgs &t, bool full) {
-  if (!full) return t.pack < 4 ? 128 : t.form == 1 ? 117 : 108;
+  if (!full) return t.pack < 4 ? 122 : t.form == 1 ? 115 : 106;
   if (t.nlev == 0) return 99;
-  return t.form == 1 ? 127 : t.form == 0 && t.emit_w[0] < 0 ? 111 : 120;
+  return t.form == 1 ? 128 : t.form == 0 && t.emit_w[0] < 0 ? 111 : 120;
 }
 
 // Column blocks, and with TT <= 0 the tile of packed delay windows, of the MBD passes of n_s series (their chunks'

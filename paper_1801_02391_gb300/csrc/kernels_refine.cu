@@ -23,7 +23,7 @@
 //    expression's; otherwise the expression is evaluated;
 //  * f0_n t_ap (u + i) is a sum of two floats, rounded under the same condition.
 // What a point contributes (du/dDM, its FP32 frequencies) is a table of the handle.  Forward and backward
-// of 200 candidates x 15 baselines x 2048 points, windows of 1 to 16 APs: 3.15 -> 0.77 ms, the same bits
+// of 200 candidates x 15 baselines x 2048 points, windows of 1 to 16 APs: 3.18 -> 0.80 ms, the same bits
 // (two baselines per CTA, to share their points' FP64: 0.85 ms, the CTAs of the longest windows end late).
 #include <climits>
 

@@ -17,7 +17,8 @@
 // form issued on few of its cycles: two serial device reads per AP, half of each CTA's threads idle).
 // Three-input maxima, a first FFT stage without its zeros and reads of two points: call 4.64 -> 4.55 ms.
 // Every sum (FFTs and windows) as packed pairs: kernel 2.98 -> 2.75 ms, call 4.40 -> 4.15 ms (the windows' sums
-// alone 2.94 ms).  Four CTAs per SM at 128 registers spill: 5.78 ms.
+// alone 2.94 ms).  Three CTAs per SM allow 168 registers, at which ptxas spills 144 to 336 bytes a thread (80 to 548 of
+// loads) beside the deep anchors that are meant to be there; four at 128 registers: 5.78 ms.
 #include "fit_common.cuh"
 #include "fft32.cuh"
 

@@ -31,7 +31,10 @@
 //          instead of 152, level 2 stays in registers.
 // Three warpgroups against two: the chain of
 // dependent work leaves issue slots free that a third warp per scheduler uses, and an A tile is read
-// by 11 CTAs instead of 16.  A search of 192 series x 20000 APs: 299.6 -> 260.5 ms.
+// by 11 CTAs instead of 16.  A search of 192 series x 20000 APs: 299.6 -> 260.5 ms.  Launches of one or two
+// rounds of CTAs take two warpgroups (plan_blocks in frbx_api.cu).  Of the instances with three, the whole-grid
+// ones of the split and E4M3 forms fit their 128 registers; ptxas spills 36 bytes a thread in the BF16 one and 106 to
+// 158 in those with delay windows (176 to 380 bytes of loads).
 // Two lower-precision forms of the same tree run one product per AP instead of three: kernel 7
 // multiplies A_hi by W_hi (BF16, about 4e-3 relative on |G|), kernel 8 multiplies E4M3 operands
 // with kind::f8f6f4 (about 6e-2 relative), A scaled per AP by the power of two s with
@@ -41,7 +44,7 @@
 // With delay search windows the SBD pass stores the rows rotated by t.rot (a multiple of 8),
 // tile row r = (m - rot) mod Ls, so the searched rows sit in the first row quarters: warps whose
 // rows are all outside the SBD window only release their slots, cells outside the windows are
-// masked, and CTAs whose 32 q lie outside the MBD window exit at once.  When the searched rows
+// masked, and CTAs whose columns lie outside the MBD window exit at once.  When the searched rows
 // fit the first 16, 32 or 64 tile rows, the SBD pass keeps only those rows of each AP, and one CTA
 // stacks the pieces of eight, four or two consecutive time tiles into its 128-row A operand: each
 // half of a row quarter's lanes, row quarter or pair of them walks its own time tile, so no epilogue
