@@ -1065,8 +1065,9 @@ int run_fit_tree(frbx_handle *h, const FitArgs &a, int nlev, int form, const int
   const size_t ser_bytes = (sizeof(int2) * std::max<size_t>(r.ser.size(), 1) + 255) & ~(size_t)255;
   FRBX_CK(h, ensure(h, h->ytree, ser_bytes + r.need()));
   int2 *d_ser = (int2 *)h->ytree.p;
+  h->ser_host = r.ser;  // kept in the handle: the copy may still be reading it when this function returns
   if (!r.ser.empty())
-    FRBX_CK(h, cudaMemcpyAsync(d_ser, r.ser.data(), sizeof(int2) * r.ser.size(), cudaMemcpyHostToDevice, st));
+    FRBX_CK(h, cudaMemcpyAsync(d_ser, h->ser_host.data(), sizeof(int2) * r.ser.size(), cudaMemcpyHostToDevice, st));
   rc = enqueue_tree(h, a, r, d_ser, (char *)h->ytree.p + ser_bytes, true, n_win, d_tab, d_tab + frbx::kMaxWin,
                     d_tab + 3 * frbx::kMaxWin, st, copied);
   // the call's stream also follows the whole copy (series that read no baseline past some b, or

@@ -317,6 +317,7 @@ struct frbx_handle {
   frbx_limits lim{};          // frbx_set_limits (all zero = defaults)
   size_t scratch_total = 0;   // bytes held by the Bufs below
   std::vector<unsigned char> dm_host;  // what the last shift table uploaded to small
+  std::vector<int2> ser_host;          // what the last window-tree fit uploaded as its series list
   const int *dk_max = nullptr;  // [n_dm] in small, of the last shift table
   Buf vis, dk, series, pnorm, stats, counts, offsets, events, small, seglist, masks, hits, errflag, refine, calib,
       ytree;
